@@ -1,0 +1,33 @@
+"""The stencil kernels' strips: row counts at and around a strip's height, widths at and around
+a warp's columns, and each side of the grid sizes at which the strip height changes, against
+the oracle's sweep (bit-exact: every step is rounded to fp32 in the stated order)."""
+import numpy as np
+import pytest
+
+import paper_2604_22228_gb300 as mpt
+import payload
+from oracle import jacobi as J
+
+pytestmark = pytest.mark.gpu
+
+VEC = [(1, 4), (1, 132), (2, 128), (2, 1028), (3, 4), (4, 124), (5, 1152), (7, 132), (767, 1024), (768, 1024), (770, 1024),
+       (4, 1 << 21), (5, 1677720), (8, 1 << 20), (9, 1048580), (2049, 4096)]
+ANY = [(1, 2), (1, 31), (2, 33), (5, 127), (64, 1023), (65, 1023), (3, 70001), (4, 129), (66, 1025), (769, 1023), (767, 1025),
+       (771, 1025), (4, 262149), (6, 131073), (1, 200003)]
+
+
+@pytest.mark.parametrize("rows,cols,offset", [(r, c, 0) for r, c in VEC] + [(r, c, 0) for r, c in ANY] +
+                         [(4, 128, 1), (771, 1024, 3), (2, 40000, 2)])
+def test_sweep_at_strip_edges(rows, cols, offset):
+    import torch
+    n = (rows + 2) * cols
+    grid = payload.fill("f32", 0x5EED0008 + rows * 131 + cols, n * 4).view(np.float32).reshape(rows + 2, cols)
+    buf_in = torch.zeros(n + offset, dtype=torch.float32, device="cuda")
+    buf_out = torch.full((n + offset + 8,), 7.0, dtype=torch.float32, device="cuda")
+    buf_in[offset:offset + n].copy_(torch.from_numpy(grid.reshape(-1)))
+    mpt.mpt_demo_jacobi_step(buf_in[offset:], buf_out[offset:], rows, cols, torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    got = buf_out[offset:offset + n].cpu().numpy().reshape(rows + 2, cols)
+    assert np.array_equal(got[1:rows + 1], J.step(grid)[1:rows + 1])
+    assert (got[0] == 7.0).all() and (got[rows + 1] == 7.0).all()  # halo rows are not written
+    assert (buf_out[:offset].cpu().numpy() == 7.0).all() and (buf_out[offset + n:].cpu().numpy() == 7.0).all()
