@@ -17,7 +17,7 @@ INCLUDE = os.path.join(ROOT, "include")
 OUT = os.path.join(PKG, "libmpt.so")
 OBJDIR = os.path.join(PKG, "_build")
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
-SOURCES = ["copy_kernels.cu", "copy_bulk.cu", "stage_consume.cu", "runtime.cu", "planner.cpp", "api_plan.cpp", "model.cpp", "tuner.cu", "batch.cu", "serve.cu", "jacobi.cu", "noalloc.cu", "host_pool.cpp", "host_probe.cpp"]
+SOURCES = ["copy_kernels.cu", "copy_bulk.cu", "hash.cu", "stage_consume.cu", "runtime.cu", "planner.cpp", "api_plan.cpp", "model.cpp", "tuner.cu", "batch.cu", "serve.cu", "jacobi.cu", "noalloc.cu", "host_pool.cpp", "host_probe.cpp"]
 
 
 def _nvcc() -> str:
@@ -28,7 +28,7 @@ def _nvcc() -> str:
 
 
 CFLAGS = [ARCH, "-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O3,-fvisibility=hidden"]
-HEADERS = ["kernels.cuh", "bulk_config.h", "batch_kernels.cuh", "copy_device.cuh", "internal.h", "ctx.h", "host_pool.h"]
+HEADERS = ["kernels.cuh", "bulk_config.h", "batch_kernels.cuh", "copy_device.cuh", "hash.cuh", "internal.h", "ctx.h", "host_pool.h"]
 STAMP = OUT + ".sha256"
 
 

@@ -8,7 +8,6 @@
 //                  message of a few MiB spreads over every SM instead of a few dozen.
 //  k_zc_copy       zero-copy kernel: the vec128 loop with plain (coherent) loads, used on
 //                  mapped page-locked host memory for host<->device transfers.
-//  k_hash          digest of a byte range (test utility).
 //
 // The bulk-copy variant of the SM copy kernel (cp.async.bulk through shared memory) is in
 // copy_bulk.cu.
@@ -131,44 +130,6 @@ __global__ void __launch_bounds__(kVecThreads) k_zc_copy(CopyArgs a) {
 __global__ void __launch_bounds__(kVecThreads) k_zc_copy_any(CopyArgs a) {
   pdl_enter();
   copy_tiles_vec<true, true, kVecUnroll>(a);
-}
-
-namespace {
-__device__ __forceinline__ uint64_t mix64(uint64_t z) {
-  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-  return z ^ (z >> 31);
-}
-}  // namespace
-
-__global__ void __launch_bounds__(256) k_hash(const uint8_t* p, uint64_t n, unsigned long long* out) {
-  constexpr uint64_t kGamma = 0x9E3779B97F4A7C15ull;
-  const uint64_t nw = (n + 7) >> 3;
-  const bool aligned = (reinterpret_cast<uintptr_t>(p) & 7) == 0;
-  uint64_t acc = 0;
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t w = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; w < nw; w += stride) {
-    uint64_t v = 0;
-    if (aligned && (w + 1) * 8 <= n) {
-      v = __ldcs(reinterpret_cast<const unsigned long long*>(p) + w);
-    } else {
-      for (int b = 0; b < 8; ++b) {
-        const uint64_t i = w * 8 + b;
-        if (i < n) v |= (uint64_t)p[i] << (8 * b);
-      }
-    }
-    acc += mix64(v ^ (w * kGamma));
-  }
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  __shared__ uint64_t warp_sum[8];
-  if ((threadIdx.x & 31) == 0) warp_sum[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint64_t s = 0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += warp_sum[i];
-    if (blockIdx.x == 0) s += mix64(n);
-    atomicAdd(out, (unsigned long long)s);
-  }
 }
 
 // ---- host side -------------------------------------------------------------------------

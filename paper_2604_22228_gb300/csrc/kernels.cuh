@@ -82,9 +82,6 @@ struct StageArgs {
 
 __global__ void k_stage_consume(StageArgs a);
 
-// ---- digest (test utility) -------------------------------------------------------
-__global__ void k_hash(const uint8_t* p, uint64_t n, unsigned long long* out);
-
 // Status codes written by kernels: (site << 8) | MPT_ETIMEDOUT.
 constexpr uint32_t kSiteBulkLoad = 1;
 constexpr uint32_t kSiteStageFlag = 2;

@@ -13,8 +13,8 @@
 // cudaGetSymbolAddress (with that device current) and cached.
 #include <mutex>
 
+#include "hash.cuh"
 #include "internal.h"
-#include "kernels.cuh"
 
 namespace {
 
@@ -69,13 +69,7 @@ extern "C" MPT_API mpt_status mpt_hash_ranges_noalloc(const void* const* ptrs, c
   // The array keeps the previous call's sums: clear the accumulators this call uses.
   e = cudaMemsetAsync(scratch, 0, n * sizeof(unsigned long long), s);
   if (e != cudaSuccess) return mpt::fail(MPT_ECUDA, "mpt_hash_ranges_noalloc: %s", cudaGetErrorString(e));
-  for (uint32_t i = 0; i < n; ++i) {
-    const uint64_t words = (nbytes[i] + 7) / 8;
-    const uint64_t want = (words + 255) / 256;
-    const uint32_t blocks = (uint32_t)(want < 1 ? 1 : (want > 4ull * (uint64_t)sms ? 4ull * (uint64_t)sms : want));
-    mpt::k_hash<<<blocks, 256, 0, s>>>(static_cast<const uint8_t*>(ptrs[i]), nbytes[i], scratch + i);
-  }
-  e = cudaGetLastError();
+  e = mpt::launch_hash(ptrs, nbytes, n, scratch, sms, s);
   if (e != cudaSuccess) return mpt::fail(MPT_ECUDA, "mpt_hash_ranges_noalloc: launch: %s", cudaGetErrorString(e));
   e = cudaMemcpyAsync(out, scratch, n * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);

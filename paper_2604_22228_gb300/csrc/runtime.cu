@@ -16,6 +16,7 @@
 #include <unordered_set>
 
 #include "ctx.h"
+#include "hash.cuh"
 
 namespace mpt {
 const char* last_error_cstr();
@@ -1269,10 +1270,7 @@ mpt_status mpt_hash_device(mpt_ctx_t c, const void* ptr, uint64_t nbytes, void* 
   CUDA_TRY(cudaSetDevice(c->device));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   CUDA_TRY(cudaMemsetAsync(c->d_hash, 0, sizeof(unsigned long long), s));
-  const uint64_t words = (nbytes + 7) / 8;
-  const uint32_t blocks = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(4ull * c->sms, (words + 255) / 256));
-  k_hash<<<blocks, 256, 0, s>>>(static_cast<const uint8_t*>(ptr), nbytes, c->d_hash);
-  CUDA_TRY(cudaGetLastError());
+  CUDA_TRY(launch_hash(&ptr, &nbytes, 1, c->d_hash, c->sms, s));
   unsigned long long h = 0;
   CUDA_TRY(cudaMemcpyAsync(&h, c->d_hash, sizeof h, cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));

@@ -1,0 +1,37 @@
+"""The digest kernel at the edges of its 16 KiB tiles and 16-byte vectors, at every alignment,
+and with more ranges than one launch takes, against the oracle's digest (whole numbers: equal)."""
+import pytest
+
+import paper_2604_22228_gb300 as mpt
+import payload
+from oracle import transfer as T
+
+pytestmark = pytest.mark.gpu
+
+TILE = 16384
+SIZES = [1, 8, 15, 16, 17, 24, 512, 513, 2047, 2048, 2049, TILE - 16, TILE - 1, TILE, TILE + 1, TILE + 17, 2 * TILE,
+         2 * TILE + 2049, 3 * TILE - 9, 40 * TILE + 5]
+
+
+@pytest.mark.parametrize("offset", list(range(16)))
+def test_tile_edges_at_every_alignment(offset):
+    import torch
+    ctx = mpt.mpt_ctx_create(0)
+    host = payload.fill("u8", 0x5EED0009 + offset, SIZES[-1] + 64)
+    t = torch.from_numpy(host).cuda()
+    got = mpt.mpt_hash_ranges_noalloc([(t.data_ptr() + offset, n) for n in SIZES])
+    want = [T.hash64(host[offset:offset + n]) for n in SIZES]
+    assert got == want
+    assert [mpt.mpt_hash_device(ctx, t.data_ptr() + offset, n) for n in SIZES] == want
+    mpt.mpt_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("n", [1, 4, 5, 159, 160, 161, 321, 1024])
+def test_many_ranges(n):
+    import torch
+    sizes = [0 if i % 7 == 3 else (i * 37) % 900 + (TILE * 3 if i % 50 == 0 else 0) for i in range(n)]
+    host = payload.fill("u8", 0x5EED000A, sum(sizes) + 16)
+    t = torch.from_numpy(host).cuda()
+    offs = [sum(sizes[:i]) for i in range(n)]
+    got = mpt.mpt_hash_ranges_noalloc([(t.data_ptr() + o, k) for o, k in zip(offs, sizes)])
+    assert got == [T.hash64(host[o:o + k]) for o, k in zip(offs, sizes)]
