@@ -13,6 +13,8 @@
 // 175 / 217, 64 registers instead of 80 173 / 277 (spills), 8 CTAs per SM 177 / 210.
 #include "hash.cuh"
 
+#include <cuda.h>
+
 #include <algorithm>
 
 #include "copy_device.cuh"
@@ -24,6 +26,12 @@ constexpr uint32_t kHashThreads = 256;
 constexpr uint32_t kHashUnroll = 4;
 constexpr uint32_t kTilePairs = kHashThreads * kHashUnroll;  // a pair: two words, 16 bytes
 constexpr uint32_t kHashCtasPerSm = 16;  // of them three resident
+// CTAs of a launch over host memory: 32 keep 1 MiB of loads in flight, enough for the host
+// link's rate, while a full grid's 15 MiB is a queue of 70 us on the link that everything else
+// crossing it waits behind (serving at 50k requests/s beside the digests of 1 % of them: p99
+// 700 us with a full grid, 235 with 32 CTAs, 283-345 with the kernel that had one 8-byte load
+// in flight per thread).
+constexpr uint32_t kHashHostCtas = 32;
 constexpr uint64_t kGamma = 0x9E3779B97F4A7C15ull;
 
 // kCap ranges by value: a launch copies its whole argument, so one range alone takes the small
@@ -180,7 +188,7 @@ __global__ void __launch_bounds__(kHashThreads, 3) k_hash(const __grid_constant_
 }
 
 template <int kCap>
-cudaError_t launch(const void* const* ptrs, const uint64_t* bytes, uint32_t n, unsigned long long* out, int sms,
+cudaError_t launch(const void* const* ptrs, const uint64_t* bytes, uint32_t n, unsigned long long* out, uint32_t ctas,
                    cudaStream_t s) {
   HashArgs<kCap> a;
   a.n = n;
@@ -196,19 +204,65 @@ cudaError_t launch(const void* const* ptrs, const uint64_t* bytes, uint32_t n, u
   for (uint32_t i = n; i <= (uint32_t)kCap; ++i) a.first_tile[i] = (uint32_t)tiles;
   a.ntiles = (uint32_t)tiles;
   if (tiles == 0) return cudaSuccess;  // empty ranges: the digest of no bytes is 0
-  const uint32_t grid = (uint32_t)std::min<uint64_t>(tiles, (uint64_t)kHashCtasPerSm * (uint32_t)sms);
-  k_hash<kCap><<<grid, kHashThreads, 0, s>>>(a);
+  k_hash<kCap><<<(uint32_t)std::min<uint64_t>(tiles, ctas), kHashThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
+
+// Memory kind of one range after another; ranges inside the allocation of the last query, the
+// usual case, are answered without another one.
+class HostSide {
+ public:
+  bool operator()(const void* p, uint64_t n) {
+    const uint64_t a = (uint64_t)(uintptr_t)p;
+    if (n == 0) return host_;
+    if (a >= lo_ && a + n <= hi_) return host_;
+    lo_ = hi_ = 0;
+    host_ = true;  // not known to CUDA: pageable host memory
+    CUmemorytype type{};
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                  CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* into[] = {&type, &base, &size};
+    static const auto query = entry();
+    if (query && query(3, what, into, (CUdeviceptr)a) == CUDA_SUCCESS && type != 0) {
+      host_ = type == CU_MEMORYTYPE_HOST;
+      if (base) {
+        lo_ = base;
+        hi_ = base + size;
+      }
+    }
+    return host_;
+  }
+
+ private:
+  using Query = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static Query entry() {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult r;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+        r != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    return reinterpret_cast<Query>(f);
+  }
+  uint64_t lo_ = 0, hi_ = 0;
+  bool host_ = true;
+};
 
 }  // namespace
 
 cudaError_t launch_hash(const void* const* ptrs, const uint64_t* bytes, uint32_t n, unsigned long long* out, int sms,
                         cudaStream_t s) {
+  HostSide host_side;
   for (uint32_t i = 0; i < n;) {
-    const uint32_t k = std::min<uint32_t>(n - i, kHashRanges);
-    const cudaError_t e = k <= 4 ? launch<4>(ptrs + i, bytes + i, k, out + i, sms, s)
-                                 : launch<kHashRanges>(ptrs + i, bytes + i, k, out + i, sms, s);
+    const bool host = host_side(ptrs[i], bytes[i]);
+    uint32_t k = 1;
+    while (i + k < n && k < (uint32_t)kHashRanges && host_side(ptrs[i + k], bytes[i + k]) == host) ++k;
+    const uint32_t ctas = host ? kHashHostCtas : kHashCtasPerSm * (uint32_t)sms;
+    const cudaError_t e = k <= 4 ? launch<4>(ptrs + i, bytes + i, k, out + i, ctas, s)
+                                 : launch<kHashRanges>(ptrs + i, bytes + i, k, out + i, ctas, s);
     if (e != cudaSuccess) return e;
     i += k;
   }

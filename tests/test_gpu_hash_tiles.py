@@ -35,3 +35,17 @@ def test_many_ranges(n):
     offs = [sum(sizes[:i]) for i in range(n)]
     got = mpt.mpt_hash_ranges_noalloc([(t.data_ptr() + o, k) for o, k in zip(offs, sizes)])
     assert got == [T.hash64(host[o:o + k]) for o, k in zip(offs, sizes)]
+
+
+def test_device_and_host_ranges_in_one_call():
+    """Ranges of device and page-locked host memory in turns: one launch for every run of
+    neighbours of one kind."""
+    import torch
+    host = payload.fill("u8", 0x5EED000B, 12 * 70000)
+    pinned = torch.from_numpy(host).pin_memory()
+    dev = pinned.cuda()
+    kinds = [0, 0, 1, 0, 1, 1, 1, 0, 0, 0, 1, 1]
+    sizes = [70000 - 13 * i if i % 5 else 0 for i in range(12)]
+    at = [(70000 * i + i) for i in range(12)]
+    got = mpt.mpt_hash_ranges_noalloc([((pinned if k else dev).data_ptr() + a, n) for k, a, n in zip(kinds, at, sizes)])
+    assert got == [T.hash64(host[a:a + n]) for a, n in zip(at, sizes)]
