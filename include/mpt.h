@@ -425,10 +425,11 @@ MPT_API mpt_status mpt_tune_get(mpt_ctx_t ctx, uint32_t dir, uint64_t nbytes, ui
 
 /* Size the context's batch ring: `slots` batches in flight at once (default 4), up to
  * `max_xfers` transfers per batch (default 4096), `ctas` CTAs of the batch kernel
- * (default 3 x SMs) and `tile_bytes` per work item (default 256 KiB; >= 4096, multiple of
- * 16).  tile_bytes is the largest tile: a batch whose kernel-moved bytes give each CTA less
- * than one tile is cut into the power of two at or above its bytes per CTA (at least
- * 32 KiB), so that a short batch spreads over the grid.  0 keeps a default.  Waits for the
+ * (default 3 x SMs; the kernel runs as many of them as are resident at once, 2 x SMs on
+ * GB300) and `tile_bytes` that a CTA moves at a time (default 256 KiB; >= 4096, multiple of
+ * 16).  A CTA's 16 warps take tiles of tile_bytes / 16 on their own.  That is the largest
+ * tile: a batch whose bytes give each warp less is cut into the power of two at or above its
+ * bytes per warp (at least 4 KiB), so that a short batch spreads over the grid.  0 keeps a default.  Waits for the
  * device; fails with EAGAIN while a batch is held.  The ring is built on first use with
  * defaults when this is never called. */
 MPT_API mpt_status mpt_batch_configure(mpt_ctx_t ctx, uint32_t slots, uint32_t max_xfers, uint32_t ctas,
@@ -479,7 +480,7 @@ MPT_API mpt_status mpt_batch_register(mpt_ctx_t ctx, const void* base, uint64_t 
 
 /* Move n transfers in one launch of the persistent batch kernel, as one replay of a slot's
  * graph on `stream` (windowed transfers, Sec. 5.3: many messages in flight, one launch).
- * The kernel's CTAs claim fixed-size tiles of the transfers through two cursors: tiles of
+ * The kernel's warps claim fixed-size tiles of the transfers through two cursors: tiles of
  * transfers with a host side (over the host link) and device-to-device tiles.  The first
  * 32 CTAs (MPT_BATCH_LINK_CTAS=k: k) start on the former and move to device tiles when they
  * run out; the others take device tiles only.  32 CTAs hold the link at its rate, and

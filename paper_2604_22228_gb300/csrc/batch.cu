@@ -3,10 +3,10 @@
 //
 // The paper's windowed benchmarks keep several messages in flight at once and find that
 // graphs pay off when many operations share one launch (Sec. 5.3, windows 1/4/16; Sec. 6).
-// Here a batch is a table of (src, dst, bytes) descriptors; the kernel's CTAs claim fixed
-// size tiles of the whole batch through one atomic cursor, so short and long messages,
+// Here a batch is a table of (src, dst, bytes) descriptors; the kernel's warps claim fixed
+// size tiles of the whole batch through atomic cursors, so short and long messages,
 // device-to-device and host<->device ones, share the SMs without per-message launches.
-// A per-descriptor tile counter detects the last tile of a message; that CTA stamps the
+// A per-transfer tile counter detects the last tile of a message; that warp stamps the
 // completion time and raises the message's flag in page-locked host memory, which is how
 // a host thread (the serving loop) sees individual messages finish while the batch runs.
 //
@@ -48,95 +48,194 @@ __device__ __forceinline__ uint64_t now_ns() {
 
 }  // namespace
 
+constexpr uint32_t kBatchThreads = 512;
+constexpr uint32_t kBatchWarps = kBatchThreads / 32;
+constexpr uint32_t kBatchCtasPerSm = 2;  // resident: 64 registers a thread
+constexpr uint32_t kLine = 128;
+
+// The work item is a warp's tile (4 to 16 KiB by default).  A batch of small transfers is
+// bound by the chain of steps around each tile (claim, search, copy, publish), a large one by
+// HBM or the host link; with a tile to a warp, no step waits for the other warps of the CTA and
+// thousands of chains run side by side.  Measured on GB300 against a tile to a CTA (claim,
+// 12-step search of two dependent loads a step, two barriers, a fence by every thread), kernel
+// time: 4096 transfers of 256 B to 64 KiB (47.5 MB) 86 us then, 25.5 now; the same off 16-byte
+// boundaries 116 and 32; 2048 of 256 B to 16 MiB on the device (3.1 GB) 935 and 917, off
+// 16-byte boundaries 1207 and 950; 512 of 256 B to 64 KiB over the link 136 and 38.
+//
+// Over the host link a row of 32 words that begins inside a 128-byte line costs a whole line
+// more: 197.6 GB/s host-to-device and 183 device-to-host with rows where the transfer puts them,
+// 210.7 and 192.8 with rows on lines of the host side, which is the link's rate (211, 193).
+//
+// Eight words a lane in flight and two CTAs per SM move 3365 GB/s of large device transfers,
+// four and three CTAs 3290; off 16-byte boundaries four words and two CTAs 3247, two words and
+// three 3035.  Tiles of 8 KiB at most 2431 GB/s (claims), 32 KiB 3301.
+
+// One warp copies n bytes s -> o: bytes until o is 16-byte aligned, 16-byte words, kU a lane
+// in flight, and the bytes left.  Rows of 32 words begin on 128-byte lines of the source
+// (src_rows) or of the destination.  Only 16-byte blocks that hold source bytes are read.
+// Without kAny the caller guarantees that s and o agree modulo 16 wherever a word is moved.
+// Loads are coherent, never through the read-only path: host memory needs that.
+template <bool kAny>
+__device__ __forceinline__ void warp_copy(const uint8_t* s, uint8_t* o, uint32_t n, bool src_rows, uint32_t lane) {
+  constexpr int kU = kAny ? 4 : 8, kRow = 32 * kU;
+  const uint32_t skew = (16u - (uint32_t)(reinterpret_cast<uintptr_t>(o) & 15)) & 15u;
+  const uint32_t head = skew < n ? skew : n;
+  if (lane < head) o[lane] = s[lane];
+  s += head;
+  o += head;
+  n -= head;
+  const int nv = (int)(n >> 4);
+  const uint32_t m = kAny ? (uint32_t)(reinterpret_cast<uintptr_t>(s) & 15) : 0u;
+  // words before the first one in its line; the first row starts there
+  int v = nv ? -(int)(((src_rows ? reinterpret_cast<uintptr_t>(s) : reinterpret_cast<uintptr_t>(o)) & (kLine - 1)) >> 4) : 0;
+  uint4* ov = reinterpret_cast<uint4*>(o) + lane;
+  if (!kAny || m == 0) {
+    const uint4* sv = reinterpret_cast<const uint4*>(s) + lane;
+    uint4 x[kU];
+    for (; v < nv; v += kRow) {
+      if (v >= 0 && v + kRow <= nv) {
+#pragma unroll
+        for (int u = 0; u < kU; ++u) x[u] = ld_once(sv + v + 32 * u);
+#pragma unroll
+        for (int u = 0; u < kU; ++u) st_plain(ov + v + 32 * u, x[u]);
+      } else {
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          const int i = v + 32 * u + (int)lane;
+          if (i >= 0 && i < nv) x[u] = ld_once(sv + v + 32 * u);
+        }
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          const int i = v + 32 * u + (int)lane;
+          if (i >= 0 && i < nv) st_plain(ov + v + 32 * u, x[u]);
+        }
+      }
+    }
+  } else {
+    // a destination word lies in two neighbouring source words, the second of them in the next
+    // lane, or for lane 31 in lane 0 of the next u; lane 31 loads the one after the last itself
+    const uint4* sw = reinterpret_cast<const uint4*>(s - m) + lane;
+    const uint32_t k = m >> 2, r = (m & 3u) * 8u;
+    for (; v < nv; v += kRow) {
+      uint4 x[kU], end = make_uint4(0, 0, 0, 0);
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const int i = v + 32 * u + (int)lane;
+        x[u] = make_uint4(0, 0, 0, 0);
+        if (i >= 0 && i <= nv) x[u] = ld_once(sw + v + 32 * u);  // word nv holds the last bytes
+      }
+      if (lane == 31 && v + kRow <= nv) end = ld_once(sw + v + kRow - 31);
+      uint4 rot = shfl4(x[0], lane + 1);
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const uint4 next = u + 1 < kU ? shfl4(x[u + 1 < kU ? u + 1 : u], lane + 1) : end;
+        const int i = v + 32 * u + (int)lane;
+        if (i >= 0 && i < nv) st_plain(ov + v + 32 * u, shift16(x[u], lane == 31 ? next : rot, k, r));
+        rot = next;
+      }
+    }
+  }
+  const uint32_t tail = ((uint32_t)nv << 4) + lane;
+  if (tail < n) o[tail] = s[tail];
+}
+
+// The last of the n descriptors from `lo` whose first tile is <= item: 32 probes a step.
+__device__ __forceinline__ uint32_t find_desc(const uint32_t* first, uint32_t lo, uint32_t n, uint32_t item,
+                                              uint32_t lane) {
+  while (n > 1) {
+    const uint32_t step = (n + 31) >> 5, i = lane * step;
+    const uint32_t c = __popc(__ballot_sync(0xffffffffu, i < n && first[lo + i] <= item)) - 1;
+    lo += c * step;
+    n = n - c * step < step ? n - c * step : step;
+  }
+  return lo;
+}
+
 template <bool kAny>
 __device__ __forceinline__ void batch_body(const BatchArgs& a) {
-  __shared__ uint32_t s_item;
   const BatchHeader h = *a.hdr;
-  const uint32_t* order = reinterpret_cast<const uint32_t*>(a.desc + h.n);
+  const BatchDesc* desc = a.desc;
+  const uint32_t* first = reinterpret_cast<const uint32_t*>(desc + h.n);
+  __shared__ uint32_t s_base;
+  const uint64_t t_start = now_ns();
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  // The CTA's class, and its first claim: as many tiles at once as spread the class evenly over
+  // its CTAs, at most one for each warp.
+  bool link = blockIdx.x < h.link_ctas && h.link_tiles > 0;
+  bool last_class = !link || h.dev_tiles == 0;
+  uint32_t lim = link ? h.link_tiles : h.dev_tiles;
+  uint32_t* cursor = link ? a.cursor : a.cursor_dev;
+  const uint32_t in_class = link ? min(h.link_ctas, gridDim.x) : gridDim.x - (h.link_tiles ? min(h.link_ctas, gridDim.x) : 0);
+  const uint32_t k0 = min(kBatchWarps, (lim + in_class - 1) / max(in_class, 1u));
+  if (threadIdx.x == 0 && k0) s_base = atomicAdd(cursor, k0);
+  __syncthreads();
+  if (warp < k0 || !last_class) {
+    uint32_t item = warp < k0 ? s_base + warp : lim;
+    while (true) {
+      if (item >= lim) {
+        if (last_class) break;
+        last_class = true;  // link tiles are gone: on to device tiles
+        link = false;
+        lim = h.dev_tiles;
+        cursor = a.cursor_dev;
+        if (lane == 0) item = atomicAdd(cursor, 1u);
+        item = __shfl_sync(0xffffffffu, item, 0);
+        continue;
+      }
+      uint32_t next = 0;
+      if (lane == 0) next = atomicAdd(cursor, 1u);  // its answer is not needed before the copy ends
+      const uint32_t pos = link ? find_desc(first, 0, h.n_link, item, lane)
+                                : find_desc(first, h.n_link, h.n - h.n_link, item, lane);
+      const BatchDesc& d = desc[pos];
+      // tiles begin on 128-byte lines of the host side, or of the destination on the device:
+      // the first one is shorter by what lies before the transfer in its line
+      const uint32_t tile = link ? h.link_tile : h.dev_tile;
+      const bool src_rows = (d.flags & (kDescHostSide | kDescHostDst)) == kDescHostSide;
+      const uint32_t lead = (uint32_t)(src_rows ? d.src : d.dst) & (kLine - 1);
+      const uint64_t end = (uint64_t)(item - d.first_tile + 1) * tile - lead, bytes = d.bytes;
+      const uint64_t off = end > tile ? end - tile : 0;
+      if (off < bytes)
+        warp_copy<kAny>(reinterpret_cast<const uint8_t*>(d.src) + off, reinterpret_cast<uint8_t*>(d.dst) + off,
+                        (uint32_t)((end < bytes ? end : bytes) - off), src_rows, lane);
+      __syncwarp();
+      if (lane == 0) {
+        // lane 0's fences cover the warp's stores, which the barrier above orders before them
+        const uint32_t idx = d.index, ntiles = d.ntiles;
+        bool last = ntiles == 1;
+        if (!last) {
+          if (d.flags & kDescHostDst) __threadfence_system();
+          uint32_t prev;
+          asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(prev) : "l"(a.done + idx) : "memory");
+          last = prev + 1 == ntiles;
+          if (last) a.done[idx] = 0;  // every tile is counted: no warp of this launch touches it again
+        }
+        if (last) {
+          a.times[idx] = now_ns();
+          // the release store's system-scope fence orders the tiles counted through `done`
+          // (each published before its count) ahead of the flag
+          asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(a.host_flags + idx), "r"(h.epoch) : "memory");
+        }
+      }
+      item = __shfl_sync(0xffffffffu, next, 0);
+    }
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
-    const uint64_t t = now_ns();
-    atomicMax(a.start_inv, ~t);
     // when the first and the last CTA of the grid started: a spread far above the launch
     // time means the grid was only partly resident (other kernels held the SMs)
-    const uint32_t k = atomicAdd(a.started, 1u);
-    if (k == 0) a.host_stamps[0] = t;
-    if (k == gridDim.x - 1) a.host_stamps[1] = t;
-  }
-  __shared__ uint32_t s_link;
-  const uint32_t dev_tiles = h.total_tiles - h.link_tiles;
-  // thread 0's claiming state: the class it claims from, and whether it has switched yet.
-  // CTAs [0, link_ctas) take link tiles first, then device tiles; the others take device
-  // tiles only.  That bounds the host-link reads and writes this launch keeps in flight,
-  // and with them the queue that every other user of the link (another batch's table copy,
-  // its completion flags, its host-side bytes) waits behind.
-  const bool may_link = blockIdx.x < h.link_ctas;
-  bool on_link = may_link && h.link_tiles > 0;
-  bool switched = !may_link;
-  while (true) {
-    if (threadIdx.x == 0) {
-      uint32_t item = ~0u;
-      while (true) {
-        const uint32_t lim = on_link ? h.link_tiles : dev_tiles;
-        if (lim) {
-          const uint32_t k = atomicAdd(on_link ? a.cursor : a.cursor_dev, 1u);
-          if (k < lim) {
-            item = k;
-            break;
-          }
-        }
-        if (switched) break;
-        switched = true;
-        on_link = !on_link;
-      }
-      s_item = item;
-      s_link = on_link ? 1u : 0u;
-    }
-    __syncthreads();
-    const uint32_t item = s_item;
-    const bool link = s_link != 0;
-    __syncthreads();
-    if (item == ~0u) break;
-    // descriptor owning this tile: within its class, the last one whose first tile is <= item
-    uint32_t lo = link ? 0 : h.n_link, hi = (link ? h.n_link : h.n_tiled) - 1;
-    while (lo < hi) {
-      const uint32_t mid = (lo + hi + 1) >> 1;
-      if (a.desc[order[mid]].first_tile <= item) lo = mid;
-      else hi = mid - 1;
-    }
-    lo = order[lo];
-    const BatchDesc d = a.desc[lo];
-    const uint64_t off = (uint64_t)(item - d.first_tile) * h.tile_bytes;
-    if (off < d.bytes) {
-      const uint64_t len = d.bytes - off < h.tile_bytes ? d.bytes - off : h.tile_bytes;
-      const uint8_t* src = reinterpret_cast<const uint8_t*>(d.src) + off;
-      uint8_t* dst = reinterpret_cast<uint8_t*>(d.dst) + off;
-      // coherent loads for every descriptor: one copy loop keeps the kernel at 40
-      // registers (three 512-thread CTAs per SM); host-memory sources need them anyway
-      cta_copy<true, kAny>(src, dst, len);
-    }
-    if (d.flags & kDescHostDst) __threadfence_system();
-    else __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      const uint32_t prev = atomicAdd(a.done + lo, 1u);
-      if (prev + 1 == d.ntiles) {
-        a.times[lo] = now_ns();
-        // the release store's system-scope fence orders the tiles counted through `done`
-        // (each published by its CTA's fence before the count) ahead of the flag
-        asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(a.host_flags + lo), "r"(h.epoch) : "memory");
-        a.done[lo] = 0;  // every tile of lo is counted: no CTA of this launch touches it again
-      }
-    }
-  }
-  if (threadIdx.x == 0) {
+    atomicMax(a.start_inv, ~t_start);
+    atomicMax(a.start_last, t_start);
     __threadfence();
-    // the last CTA out: every CTA has stopped claiming, so the cursors and the start
-    // counters can go back to zero for the slot's next launch
+    // the last CTA out: every warp has stopped claiming, so the cursors can go back to zero
+    // for the slot's next launch
     if (atomicAdd(a.exited, 1u) == gridDim.x - 1) {
-      *a.start_out = atomicExch(a.start_inv, 0ull);
+      __threadfence();
+      const unsigned long long inv = atomicExch(a.start_inv, 0ull);
+      *a.start_out = inv;
+      a.host_stamps[0] = ~inv;
+      a.host_stamps[1] = atomicExch(a.start_last, 0ull);
       *a.cursor = 0;
       *a.cursor_dev = 0;
-      *a.started = 0;
       __threadfence();
       *a.exited = 0;
     }
@@ -153,21 +252,30 @@ __global__ void k_batch_dma_done(BatchArgs a, const uint32_t* dma_map, uint32_t 
   asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(a.host_flags + idx), "r"(a.hdr->epoch) : "memory");
 }
 
-__global__ void __launch_bounds__(kVecThreads, 3) k_batch(BatchArgs a) { batch_body<false>(a); }
-__global__ void __launch_bounds__(kVecThreads) k_batch_any(BatchArgs a) { batch_body<true>(a); }
+__global__ void __launch_bounds__(kBatchThreads, kBatchCtasPerSm) k_batch(BatchArgs a) { batch_body<false>(a); }
+__global__ void __launch_bounds__(kBatchThreads, kBatchCtasPerSm) k_batch_any(BatchArgs a) { batch_body<true>(a); }
 
 namespace {
 
 constexpr uint32_t kDefaultSlots = 4;
 constexpr uint32_t kDefaultMaxXfers = 4096;
 constexpr uint32_t kDefaultTile = 256 * 1024;
-constexpr uint64_t kMinAdaptiveTile = 32 * 1024;  // smallest tile a short batch is cut into
-// CTAs of a launch that may take link tiles (MPT_BATCH_LINK_CTAS overrides).  32 CTAs keep
-// 1 MiB of host-link traffic in flight, about 5 us of the link: enough to hold it at its
-// rate (host-to-device 204 GB/s, device-to-host 176 GB/s, as with every CTA), while a longer
-// queue only delays whatever else crosses the link
+constexpr uint32_t kMinTile = 4 * 1024;  // smallest tile a short batch is cut into
+// CTAs of a launch that may take link tiles (MPT_BATCH_LINK_CTAS overrides).  32 CTAs keep at
+// most 2 MiB of host-link traffic in flight, about 10 us of the link.  512 transfers of 256 B
+// to 4 MiB with 8 / 16 / 32 / 48 such CTAs: all host-to-device 209 / 210 / 211 / 211 GB/s, all
+// device-to-host 153 / 192 / 193 / 193, half and half 181 / 237 / 266 / 288; a longer queue
+// only delays whatever else crosses the link (serving at 50k requests/s, p99 with 24 / 32 / 48:
+// 277 / 290 / 333 us)
 constexpr uint32_t kDefaultLinkCtas = 32;
 constexpr uint32_t kDmaDirs = 3;  // lanes per direction: D2D, H2D, D2H
+
+// CTAs of a batch kernel: the configured ones (by default 3 per SM), as far as they are
+// resident at once.
+uint32_t grid_ctas(mpt_ctx_t c) {
+  const uint32_t sms = (uint32_t)c->sms;
+  return std::min(c->batch_ctas ? c->batch_ctas : 3u * sms, kBatchCtasPerSm * sms);
+}
 
 uint64_t host_ns() {
   return (uint64_t)std::chrono::duration_cast<std::chrono::nanoseconds>(
@@ -196,7 +304,7 @@ mpt_status slot_init(mpt_ctx_t c, BatchSlot& s, uint32_t max_xfers, uint32_t cta
   s.dma_lanes = c->batch_dma_lanes;
   s.dma_items = c->batch_dma_lanes ? c->batch_dma_items : 0;
   const uint32_t ndma = kDmaDirs * s.dma_lanes * s.dma_items;
-  // table: header | lane map[ndma] | desc[n] | order[n] (BatchArgs): a batch copies its first
+  // table: header | lane map[ndma] | desc[n] | first[n] (BatchArgs): a batch copies its first
   // desc_off + n * 44 bytes
   const size_t map_off = sizeof(BatchHeader);
   s.desc_off = (map_off + (size_t)ndma * sizeof(uint32_t) + 15) & ~(size_t)15;
@@ -226,12 +334,12 @@ mpt_status slot_init(mpt_ctx_t c, BatchSlot& s, uint32_t max_xfers, uint32_t cta
   s.args.hdr = reinterpret_cast<const BatchHeader*>(s.d_table);
   s.args.desc = reinterpret_cast<const BatchDesc*>(s.d_table + s.desc_off);
   s.args.cursor = reinterpret_cast<uint32_t*>(s.d_ctrl);
-  s.args.cursor_dev = reinterpret_cast<uint32_t*>(s.d_ctrl + 24);
+  s.args.cursor_dev = reinterpret_cast<uint32_t*>(s.d_ctrl + 128);
   s.args.start_inv = reinterpret_cast<unsigned long long*>(s.d_ctrl + 8);
+  s.args.start_last = reinterpret_cast<unsigned long long*>(s.d_ctrl + 16);
   s.args.start_out = reinterpret_cast<unsigned long long*>(s.d_ctrl + 32);
   s.args.done = reinterpret_cast<uint32_t*>(s.d_ctrl + 256);
-  s.args.started = reinterpret_cast<uint32_t*>(s.d_ctrl + 16);
-  s.args.exited = reinterpret_cast<uint32_t*>(s.d_ctrl + 20);
+  s.args.exited = reinterpret_cast<uint32_t*>(s.d_ctrl + 24);
   CUDA_TRY(cudaHostAlloc(reinterpret_cast<void**>(&s.h_stamps), 2 * sizeof(unsigned long long),
                          cudaHostAllocMapped | cudaHostAllocPortable));
   s.h_stamps[0] = s.h_stamps[1] = 0;
@@ -253,9 +361,8 @@ mpt_status slot_init(mpt_ctx_t c, BatchSlot& s, uint32_t max_xfers, uint32_t cta
     void* params[] = {&s.args};
     cudaKernelNodeParams kp{};
     kp.func = gi == 0 ? reinterpret_cast<void*>(&k_batch) : reinterpret_cast<void*>(&k_batch_any);
-    // the general kernel holds two CTAs per SM (64 registers): keep all of them resident
-    kp.gridDim = dim3(gi == 0 ? ctas : std::min<uint32_t>(ctas, 2u * (uint32_t)c->sms));
-    kp.blockDim = dim3(kVecThreads);
+    kp.gridDim = dim3(ctas);
+    kp.blockDim = dim3(kBatchThreads);
     kp.kernelParams = params;
     CUDA_TRY(cudaGraphAddKernelNode(&kn, s.graph[gi], deps, 1, &kp));
     // DMA lanes beside the kernel: per direction, chains of memcpy -> completion kernel.
@@ -333,9 +440,7 @@ mpt_status batch_setup(mpt_ctx_t c) {
   const uint32_t nslots = c->batch_slots ? c->batch_slots
                                          : (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(64, env_or("MPT_BATCH_SLOTS", kDefaultSlots)));
   const uint32_t maxx = c->batch_max_xfers ? c->batch_max_xfers : kDefaultMaxXfers;
-  // three 512-thread CTAs per SM (the aligned kernel's register limit): high occupancy,
-  // which the latency of host-link reads needs; all CTAs resident at once
-  const uint32_t ctas = c->batch_ctas ? c->batch_ctas : 3u * (uint32_t)c->sms;
+  const uint32_t ctas = grid_ctas(c);
   if (!c->batch_tile) c->batch_tile = kDefaultTile;
   c->batch_split = env_or("MPT_BATCH_SPLIT", 1) != 0;
   c->batch_link_ctas = (uint32_t)env_or("MPT_BATCH_LINK_CTAS", 0);
@@ -583,9 +688,6 @@ mpt_status mpt_batch_submit(mpt_ctx_t c, const mpt_xfer* xfers, size_t n, void* 
   CUDA_TRY(cudaEventSynchronize(s.done_ev));
   s.epoch++;
   if (s.epoch == 0) s.epoch = 1;
-  BatchHeader* h = reinterpret_cast<BatchHeader*>(s.h_table);
-  BatchDesc* d = reinterpret_cast<BatchDesc*>(s.h_table + s.desc_off);
-  uint32_t* order = reinterpret_cast<uint32_t*>(d + n);
   // DMA lanes: largest eligible entries first, each to the least-loaded lane of its
   // direction with a free item (longest-processing-time order); the rest stay with the kernel
   const uint32_t ndma = kDmaDirs * s.dma_lanes * s.dma_items;
@@ -611,59 +713,55 @@ mpt_status mpt_batch_submit(mpt_ctx_t c, const mpt_xfer* xfers, size_t n, void* 
       to_dma[i] = 1;
     }
   }
-  // tiles numbered within two classes, link (a host side) and device, each descriptor's
-  // tiles contiguous in its class; order lists the descriptors with tiles, link class first
+  // two classes of tiles, link (a host side) and device; one class when the split is off
+  const auto cls_of = [&](const mpt_xfer& x) { return (c->batch_split && x.dir == MPT_D2D) ? 1 : 0; };
   bool any_shift = false;
-  uint64_t kernel_bytes = 0;
+  uint64_t cls_bytes[2] = {0, 0};
+  uint32_t cls_n[2] = {0, 0};
   for (size_t i = 0; i < n; ++i) {
     if (to_dma[i]) continue;
     const mpt_xfer& x = xfers[i];
     any_shift |= (((uintptr_t)x.src ^ (uintptr_t)x.dst) & 15) != 0 && x.bytes >= 16;
-    kernel_bytes += x.bytes;
+    cls_bytes[cls_of(x)] += x.bytes;
+    cls_n[cls_of(x)]++;
   }
   const int gi = any_shift ? 1 : 0;
-  const uint32_t ctas = c->batch_ctas ? c->batch_ctas : 3u * (uint32_t)c->sms;
-  const uint32_t grid = gi == 0 ? ctas : std::min<uint32_t>(ctas, 2u * (uint32_t)c->sms);  // as slot_init
-  // tile size: the configured one, unless the batch is too small to give every CTA a full
-  // tile; then the power of two at or above the kernel's bytes per CTA, at least 32 KiB (a
-  // CTA moves 32 KiB per round of loads), so that a short batch spreads over the grid
-  // instead of queueing its bytes behind a few CTAs
-  uint64_t tile = c->batch_tile;
-  {
-    const uint64_t per_cta = (kernel_bytes + grid - 1) / grid;
-    uint64_t t = kMinAdaptiveTile;
-    while (t < per_cta && t < tile) t <<= 1;  // bounded by the configured tile: no overflow
-    tile = std::min<uint64_t>(tile, t);
+  const uint32_t ctas = grid_ctas(c);
+  uint32_t link_ctas = 0;
+  if (cls_n[0]) link_ctas = c->batch_split ? std::min(ctas, c->batch_link_ctas ? c->batch_link_ctas : kDefaultLinkCtas) : ctas;
+  // tile size of each class: a warp's part of the configured tile, unless the class is too small
+  // to give every warp a full one; then the power of two at or above its bytes per warp
+  const uint32_t max_tile = std::max<uint32_t>(256, c->batch_tile / kBatchWarps / kLine * kLine);
+  uint32_t tile[2];
+  for (int k = 0; k < 2; ++k) {
+    const uint64_t warps = (uint64_t)kBatchWarps * (k == 0 ? link_ctas : std::max(1u, ctas - link_ctas));
+    uint64_t t = kMinTile;
+    while (t < max_tile && t * warps < cls_bytes[k]) t <<= 1;
+    tile[k] = (uint32_t)std::min<uint64_t>(max_tile, t);
   }
-  uint64_t tiles[2] = {0, 0};  // [0] link, [1] device
-  uint32_t n_link = 0, n_dev = 0;
+  const uint32_t n_tiled = cls_n[0] + cls_n[1];
+  BatchHeader* h = reinterpret_cast<BatchHeader*>(s.h_table);
+  BatchDesc* d = reinterpret_cast<BatchDesc*>(s.h_table + s.desc_off);
+  uint32_t* first = reinterpret_cast<uint32_t*>(d + n_tiled);
+  uint64_t tiles[2] = {0, 0};
+  uint32_t at[2] = {0, cls_n[0]};
   for (size_t i = 0; i < n; ++i) {
+    if (to_dma[i]) continue;
     const mpt_xfer& x = xfers[i];
-    const uint32_t fl = (x.dir == MPT_D2H ? kDescHostDst : 0u) | (x.dir != MPT_D2D ? kDescHostSide : 0u) |
-                        (to_dma[i] ? kDescDma : 0u);
-    const uint64_t t = to_dma[i] ? 0 : std::max<uint64_t>(1, (x.bytes + tile - 1) / tile);
-    // one class for everything when the split is off
-    const int cls = (c->batch_split && x.dir == MPT_D2D) ? 1 : 0;
-    d[i] = BatchDesc{(uint64_t)(uintptr_t)x.src, (uint64_t)(uintptr_t)x.dst, x.bytes, (uint32_t)tiles[cls],
-                     (uint32_t)t, fl, 0u};
-    tiles[cls] += t;
-    if (t) (cls ? n_dev : n_link)++;
+    const int k = cls_of(x);
+    const uint32_t fl = (x.dir == MPT_D2H ? kDescHostDst : 0u) | (x.dir != MPT_D2D ? kDescHostSide : 0u);
+    const uint64_t lead = (uintptr_t)(x.dir == MPT_H2D ? x.src : x.dst) & (kLine - 1);
+    const uint64_t t = std::max<uint64_t>(1, (x.bytes + lead + tile[k] - 1) / tile[k]);
+    first[at[k]] = (uint32_t)tiles[k];
+    d[at[k]++] = BatchDesc{(uint64_t)(uintptr_t)x.src, (uint64_t)(uintptr_t)x.dst, x.bytes, (uint32_t)tiles[k],
+                           (uint32_t)t, fl, (uint32_t)i};
+    tiles[k] += t;
   }
-  if (tiles[0] + tiles[1] >= (1ull << 32))
+  // (every warp claims once past the end: the cursors need that much room)
+  if (std::max(tiles[0], tiles[1]) >= (1ull << 32) - (1ull << 28))
     return fail(MPT_EINVAL, "mpt_batch_submit: batch too large for 32-bit tile indices");
-  {
-    uint32_t li = 0, di = n_link;
-    for (size_t i = 0; i < n; ++i) {
-      if (!d[i].ntiles) continue;
-      const bool dev = c->batch_split && xfers[i].dir == MPT_D2D;
-      order[dev ? di++ : li++] = (uint32_t)i;
-    }
-  }
-  uint32_t link_ctas = grid;  // split off: one class, every CTA on it
-  if (c->batch_split && tiles[0])
-    link_ctas = std::min(grid, c->batch_link_ctas ? c->batch_link_ctas : kDefaultLinkCtas);
-  *h = BatchHeader{(uint32_t)n, (uint32_t)(tiles[0] + tiles[1]), (uint32_t)tile, s.epoch,
-                   (uint32_t)tiles[0], n_link, n_link + n_dev, link_ctas};
+  link_ctas = (uint32_t)std::min<uint64_t>(link_ctas, tiles[0]);
+  *h = BatchHeader{n_tiled, cls_n[0], (uint32_t)tiles[0], (uint32_t)tiles[1], tile[0], tile[1], s.epoch, link_ctas};
   for (uint32_t k = 0; k < ndma; ++k) {  // retarget used lane items, switch the rest off
     const uint32_t i = s.h_dma_map[k];
     const uint8_t want = i != ~0u;

@@ -19,43 +19,44 @@ constexpr uint32_t kDescDma = 4;       // moved by a copy-engine lane, not by th
 // mixed batch, stays busy from the start while the device tiles run beside it, and no more
 // of its traffic is in flight than the link group keeps there.
 struct BatchHeader {
-  uint32_t n;            // descriptors in this batch
-  uint32_t total_tiles;  // sum of tiles over descriptors, both classes
-  uint32_t tile_bytes;
+  uint32_t n;            // descriptors with tiles: link class first, then the device class
+  uint32_t n_link;       // of them in the link class
+  uint32_t link_tiles;   // tiles of each class
+  uint32_t dev_tiles;
+  uint32_t link_tile;    // bytes of a tile of each class
+  uint32_t dev_tile;
   uint32_t epoch;        // value written to a finished descriptor's host flag
-  uint32_t link_tiles;   // tiles of the link class (the rest are device tiles)
-  uint32_t n_link;       // descriptors with tiles in the link class: order[0, n_link)
-  uint32_t n_tiled;      // descriptors with tiles: order[n_link, n_tiled) are the device class
   uint32_t link_ctas;    // CTAs that may take link tiles (the first ones of the grid)
 };
 
 struct BatchDesc {
   uint64_t src, dst, bytes;
   uint32_t first_tile;  // prefix sum of tiles before this descriptor, within its class
-  uint32_t ntiles;      // max(1, ceil(bytes / tile)); 0 for a descriptor a DMA lane moves
+  uint32_t ntiles;      // max(1, ceil(bytes / tile))
   uint32_t flags;
-  uint32_t pad;
+  uint32_t index;       // the transfer's place in the caller's batch: its flag, count and time
 };
 
-// Device table of one batch, packed so that a batch of n descriptors is one copy of its
-// first bytes: header | DMA-lane map | desc[n] | order[n], where order lists the
-// descriptors with tiles, link class first (its address follows from n).
+// Device table of one batch, packed so that a batch of n transfers is one copy of its first
+// bytes: header | DMA-lane map | desc[n] | first[n], where first repeats the descriptors'
+// first_tile for the search (its address follows from hdr->n; transfers of a DMA lane have no
+// descriptor).
 //
-// The launch counters (cursors, per-descriptor tile counts, started and exited CTAs, the
-// start time) are zero when a launch begins and the kernel leaves them zero: the CTA that
-// counts a descriptor's last tile clears that descriptor's count, and the last CTA to exit,
-// once no CTA can claim any more, clears the rest.  No reset node runs between launches.
+// The launch counters (cursors, per-transfer tile counts, exited CTAs, start times) are zero
+// when a launch begins and the kernel leaves them zero: the warp that counts a transfer's last
+// tile clears that transfer's count, and the last CTA to exit, once no warp can claim any
+// more, clears the rest.  No reset node runs between launches.
 struct BatchArgs {
   const BatchHeader* hdr;
-  const BatchDesc* desc;         // desc[0..n); order[0..n) follows it
+  const BatchDesc* desc;
   uint32_t* cursor;              // next link tile to claim
   uint32_t* cursor_dev;          // next device tile to claim
-  unsigned long long* start_inv; // ~(kernel start time), max over CTAs, during a launch
+  unsigned long long* start_inv; // ~(first CTA's start time) while CTAs exit
+  unsigned long long* start_last;  // last CTA's start time while CTAs exit
   unsigned long long* start_out; // the launch's ~(start time), kept after the launch
-  uint32_t* done;                // tiles finished per descriptor
-  unsigned long long* times;     // completion time per descriptor (global timer, ns)
-  uint32_t* host_flags;          // device alias of page-locked flags, one per descriptor
-  uint32_t* started;             // CTAs that have started
+  uint32_t* done;                // tiles finished per transfer
+  unsigned long long* times;     // completion time per transfer (global timer, ns)
+  uint32_t* host_flags;          // device alias of page-locked flags, one per transfer
   uint32_t* exited;              // CTAs that have stopped claiming
   unsigned long long* host_stamps;  // device alias of page-locked [first, last] CTA start times
 };
@@ -64,8 +65,8 @@ struct BatchArgs {
 // moved (~0 when the item is unused); stamps its time and raises its host flag.
 __global__ void k_batch_dma_done(BatchArgs a, const uint32_t* dma_map, uint32_t item);
 
-// k_batch needs every descriptor's source and destination to agree modulo 16;
-// k_batch_any copies any alignment.
+// k_batch needs every transfer's source and destination to agree modulo 16; k_batch_any copies
+// any alignment.
 __global__ void k_batch(BatchArgs a);
 __global__ void k_batch_any(BatchArgs a);
 

@@ -51,6 +51,15 @@ __device__ __forceinline__ uint4 ld_plain(const uint4* p) {
   return v;
 }
 
+// Coherent as ld_plain, for bytes that are read once: not kept in L1.
+__device__ __forceinline__ uint4 ld_once(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
+}
+
 __device__ __forceinline__ void st_plain(uint4* p, const uint4& v) {
   asm volatile("st.global.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
                : "memory");
@@ -73,6 +82,11 @@ __device__ __forceinline__ void copy_edges(const uint8_t* s, uint8_t* o, const R
   const uint64_t tail_start = d.head + body_bytes;
   const uint32_t tail = (uint32_t)(d.bytes - tail_start);
   if (tid >= 32 && tid < 32 + tail) o[tail_start + (tid - 32)] = s[tail_start + (tid - 32)];
+}
+
+__device__ __forceinline__ uint4 shfl4(const uint4& v, uint32_t from) {
+  return make_uint4(__shfl_sync(0xffffffffu, v.x, from), __shfl_sync(0xffffffffu, v.y, from),
+                    __shfl_sync(0xffffffffu, v.z, from), __shfl_sync(0xffffffffu, v.w, from));
 }
 
 // Bytes [4k + r/8, 4k + r/8 + 16) of the 32-byte little-endian concatenation w0 | w1

@@ -74,11 +74,6 @@ __device__ __forceinline__ TileVecs load_tile(const uint4* v, bool last_lane) {
   return t;
 }
 
-__device__ __forceinline__ uint4 shfl4(const uint4& v, uint32_t from) {
-  return make_uint4(__shfl_sync(0xffffffffu, v.x, from), __shfl_sync(0xffffffffu, v.y, from),
-                    __shfl_sync(0xffffffffu, v.z, from), __shfl_sync(0xffffffffu, v.w, from));
-}
-
 // Pair u of this lane.  Off a 16-byte boundary a pair lies in two neighbouring vectors, the
 // second of them in the next lane, or for lane 31 in lane 0 of the next u.
 template <bool kShift>
