@@ -60,6 +60,33 @@ __device__ __forceinline__ uint4 ld_once(const uint4* p) {
   return v;
 }
 
+// 32 bytes in one instruction, for both ends 32-byte aligned.
+struct Wide {
+  uint32_t w[8];
+};
+
+template <bool kCoherent>
+__device__ __forceinline__ Wide ld_wide(const void* p) {
+  Wide v;
+  if (kCoherent)
+    asm volatile("ld.global.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3]), "=r"(v.w[4]), "=r"(v.w[5]), "=r"(v.w[6]),
+                   "=r"(v.w[7])
+                 : "l"(p));
+  else
+    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3]), "=r"(v.w[4]), "=r"(v.w[5]), "=r"(v.w[6]),
+                   "=r"(v.w[7])
+                 : "l"(p));
+  return v;
+}
+
+__device__ __forceinline__ void st_wide(void* p, const Wide& v) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(v.w[0]), "r"(v.w[1]), "r"(v.w[2]),
+               "r"(v.w[3]), "r"(v.w[4]), "r"(v.w[5]), "r"(v.w[6]), "r"(v.w[7])
+               : "memory");
+}
+
 __device__ __forceinline__ void st_plain(uint4* p, const uint4& v) {
   asm volatile("st.global.v4.u32 [%0], {%1,%2,%3,%4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
                : "memory");
@@ -74,7 +101,7 @@ __device__ __forceinline__ int find_range(const Args& a, uint32_t t) {
 }
 
 // Head (bytes before the destination-aligned body) and tail (bytes after it) of a range;
-// threads 0..15 copy the head, threads 32..47 the tail (blocks of at least 48 threads).
+// threads 0..31 copy the head, threads 32..63 the tail (of at most 31 bytes each).
 template <typename Range>
 __device__ __forceinline__ void copy_edges(const uint8_t* s, uint8_t* o, const Range& d, uint64_t body_bytes) {
   const uint32_t tid = threadIdx.x;

@@ -9,15 +9,14 @@ namespace mpt {
 // ---- byte-range copies (SM copy kernel, zero-copy kernel) ------------------------
 
 constexpr int kInlineRanges = 16;     // ranges carried by value in one launch
-constexpr int kVecThreads = 512;      // vec128 kernel block size
-constexpr int kVecUnroll = 8;         // 16-byte vectors in flight per thread per tile
-constexpr uint64_t kVecTileVecs = (uint64_t)kVecThreads * kVecUnroll;  // 64 KiB tiles
+constexpr int kVecThreads = 512;      // block size of the vector copy kernels
+constexpr uint32_t kVecTile = kVecThreads * 32;  // tile bytes at one 32-byte load per thread
 constexpr int kBulkThreads = 64;      // bulk kernel block: a producer warp and a consumer warp
 
 // One contiguous range to copy: src + src_off -> dst + dst_off, `bytes` long.
-// head: bytes copied singly until the destination is 16-byte aligned; shift: the source
-// address modulo 16 after the head -- 0 when source and destination agree modulo 16, else
-// each 16-byte destination word is assembled from two aligned source words.
+// head: bytes copied singly until the destination is aligned to a unit, 32 bytes for the vector
+// kernels and 16 for the bulk kernel; shift: source minus destination address modulo a unit -- 0
+// when they agree, else each destination unit is assembled from two source units.
 struct RangeDesc {
   uint64_t src_off;
   uint64_t dst_off;
@@ -26,35 +25,35 @@ struct RangeDesc {
   uint32_t shift;
 };
 
-struct CopyArgs {
+// A launch's arguments: up to kN ranges by value.
+template <int kN>
+struct CopyArgsT {
   const uint8_t* src;
   uint8_t* dst;
-  uint32_t any_shift;                    // some range has shift != 0: launch an *_any kernel
+  uint32_t* status;                      // device status word (bounded waits)
+  uint32_t any_shift;                    // vector kernels: some range has shift != 0
+  uint32_t src_lines;                    // tiles begin on lines of the source, not of the destination
   uint32_t nranges;
   uint32_t ntiles;                       // sum of tiles over ranges
-  uint32_t tile_start[kInlineRanges + 1];
-  RangeDesc r[kInlineRanges];
-  uint32_t* status;                      // device status word (bounded waits)
   uint32_t bulk_cfg;                     // bulk variant: index into the bulk configurations
-  uint32_t piece;                        // bulk variant: tile bytes (that configuration's stage)
+  uint32_t piece;                        // tile bytes
+  uint32_t tile_start[kN + 1];
+  RangeDesc r[kN];
 };
+using CopyArgs = CopyArgsT<kInlineRanges>;
 
 // Fill `a` for up to kInlineRanges ranges with the tiling of `variant` (0 vec128,
-// 1 bulk in configuration bulk_cfg (bulk_config.h), 2 zero-copy, 3 vec128 with 8 KiB tiles).  Returns
-// kArgsOk, kArgsNeedVec when a bulk launch must fall back to vec128 (source and destination
-// differ modulo 16, which cp.async.bulk cannot copy), or kArgsTooLarge.
+// 1 bulk in configuration bulk_cfg (bulk_config.h), 2 zero-copy, 3 vec128 with its smallest tiles)
+// for a grid of at most `ctas` on `sms` SMs.  src_lines: the source is the host side of a
+// zero-copy launch.  Returns kArgsOk, kArgsNeedVec when a bulk launch must fall back to vec128
+// (source and destination differ modulo 16, which cp.async.bulk cannot copy), or kArgsTooLarge.
 constexpr int kArgsOk = 0, kArgsNeedVec = 1, kArgsTooLarge = 2;
-int make_copy_args(CopyArgs& a, const void* src, void* dst, const RangeDesc* ranges, int n,
-                   int variant, uint32_t* status, uint32_t bulk_cfg);
+int make_copy_args(CopyArgs& a, const void* src, void* dst, const RangeDesc* ranges, int n, int variant,
+                   uint32_t* status, uint32_t bulk_cfg, uint32_t ctas, uint32_t sms, bool src_lines);
 
-// *_any variants also copy ranges whose source and destination differ modulo 16
-// (RangeDesc.shift != 0); the plain ones are leaner and need every shift to be 0.
-__global__ void k_sm_copy_vec(CopyArgs a);
-__global__ void k_sm_copy_vec_any(CopyArgs a);
-__global__ void k_sm_copy_vec8k(CopyArgs a);
-__global__ void k_sm_copy_vec8k_any(CopyArgs a);
-__global__ void k_zc_copy(CopyArgs a);
-__global__ void k_zc_copy_any(CopyArgs a);
+// The vector copy kernel for `a` (variant 0, 2 or 3): with a.nranges == 1 it takes a
+// CopyArgsT<1>, otherwise a CopyArgs.
+void* vec_copy_fn(const CopyArgs& a, bool zero_copy);
 
 // ---- flag-chained stage consumer (host-to-device staged path) ----------------------
 // The copy engine fills stage chunk k and a memset node then sets ready[k] = 1.  The
@@ -74,11 +73,13 @@ struct StageArgs {
   uint32_t* ready;           // nchunks flags
   uint32_t* done;            // nchunks tile counters
   uint32_t nchunks;
-  uint32_t tiles_per_chunk;  // ceil(max chunk bytes / tile)
+  uint32_t tiles_per_chunk;  // ceil(max chunk bytes / kStageTile)
   uint32_t* status;
   uint64_t timeout_ns;       // wait limit per chunk flag when wait_ns is null
   const uint64_t* wait_ns;   // the context's wait-limit word (device memory), read at each wait
 };
+
+constexpr uint32_t kStageTile = 64 * 1024;
 
 __global__ void k_stage_consume(StageArgs a);
 

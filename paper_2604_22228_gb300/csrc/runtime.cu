@@ -126,22 +126,38 @@ std::vector<RangeDesc> path_ranges(const mpt_plan_s* plan, uint32_t p) {
   return out;
 }
 
-void* kernel_fn(int variant, bool any_shift, uint32_t bulk_cfg) {
-  if (variant == 1) return const_cast<void*>(bulk_config(bulk_cfg).fn);
-  if (variant == 2) return any_shift ? reinterpret_cast<void*>(&k_zc_copy_any) : reinterpret_cast<void*>(&k_zc_copy);
-  if (variant == 3)
-    return any_shift ? reinterpret_cast<void*>(&k_sm_copy_vec8k_any) : reinterpret_cast<void*>(&k_sm_copy_vec8k);
-  return any_shift ? reinterpret_cast<void*>(&k_sm_copy_vec_any) : reinterpret_cast<void*>(&k_sm_copy_vec);
+void* kernel_fn(int variant, const CopyArgs& a) {
+  return variant == 1 ? const_cast<void*>(bulk_config(a.bulk_cfg).fn) : vec_copy_fn(a, variant == 2);
 }
 
-// Build CopyArgs for up to kInlineRanges ranges; the bulk variant falls back to vec128
-// when a range's source and destination differ modulo 16.
-mpt_status prepare_copy(CopyArgs& a, int& variant, const void* src, void* dst, const RangeDesc* r, int n,
-                        uint32_t* status, uint32_t bulk_cfg = kBulkDefaultConfig) {
-  int rc = make_copy_args(a, src, dst, r, n, variant, status, bulk_cfg);
+// A launch's argument block: the vector kernels take a single range alone, in fewer bytes.
+struct CopyParams {
+  CopyArgsT<1> one;
+  void* p[1];
+  CopyParams(int variant, CopyArgs& a) {
+    p[0] = &a;
+    if (variant == 1 || a.nranges != 1) return;
+    one = CopyArgsT<1>{a.src, a.dst, a.status, a.any_shift, a.src_lines, 1, a.ntiles, a.bulk_cfg, a.piece,
+                       {0, a.tile_start[1]}, {a.r[0]}};
+    p[0] = &one;
+  }
+};
+
+// Build CopyArgs for up to kInlineRanges ranges and a grid of at most `ctas` (0: the default of the
+// path kind); the bulk variant falls back to vec128 when a range's source and destination differ
+// modulo 16.  src_lines: see make_copy_args.
+mpt_status prepare_copy(mpt_ctx_t c, CopyArgs& a, int& variant, const void* src, void* dst, const RangeDesc* r, int n,
+                        uint32_t& ctas, bool src_lines = false) {
+  const bool dflt = ctas == 0;
+  const auto grid = [&] {
+    if (dflt) ctas = default_ctas(c, variant == 2 ? MPT_PATH_ZC : MPT_PATH_SM, (uint32_t)variant);
+  };
+  grid();
+  int rc = make_copy_args(a, src, dst, r, n, variant, c->d_status, c->bulk_cfg, ctas, (uint32_t)c->sms, src_lines);
   if (rc == kArgsNeedVec) {
     variant = 0;
-    rc = make_copy_args(a, src, dst, r, n, variant, status, bulk_cfg);
+    grid();
+    rc = make_copy_args(a, src, dst, r, n, variant, c->d_status, c->bulk_cfg, ctas, (uint32_t)c->sms, src_lines);
   }
   if (rc != kArgsOk) return fail(MPT_EINVAL, "copy of more than 2^31 tiles");
   return MPT_OK;
@@ -161,13 +177,13 @@ size_t smem_for(int variant, const CopyArgs& a) {
 mpt_status add_copy_node(cudaGraph_t g, const cudaGraphNode_t* deps, size_t ndeps, cudaGraphNode_t* node,
                          int variant, const CopyArgs& a, uint32_t ctas, mpt_graph_info& info) {
   CopyArgs args = a;
-  void* params[] = {&args};
+  CopyParams params(variant, args);
   cudaKernelNodeParams kp{};
-  kp.func = kernel_fn(variant, a.any_shift != 0, a.bulk_cfg);
+  kp.func = kernel_fn(variant, a);
   kp.gridDim = grid_for(a, ctas);
   kp.blockDim = dim3(block_for(variant));
   kp.sharedMemBytes = (unsigned)smem_for(variant, a);
-  kp.kernelParams = params;
+  kp.kernelParams = params.p;
   CUDA_TRY(cudaGraphAddKernelNode(node, g, deps, ndeps, &kp));
   info.kernel_nodes++;
   return MPT_OK;
@@ -177,11 +193,11 @@ mpt_status add_copy_node(cudaGraph_t g, const cudaGraphNode_t* deps, size_t ndep
 // the end of a copy kernel before it on the stream (the kernels wait for that kernel's
 // completion before touching memory).  Not used inside a stream capture.
 mpt_status launch_copy(cudaStream_t s, int variant, const CopyArgs& a, uint32_t ctas, bool pdl = false) {
-  void* kfn = kernel_fn(variant, a.any_shift != 0, a.bulk_cfg);
+  void* kfn = kernel_fn(variant, a);
   CopyArgs args = a;
-  void* params[] = {&args};
+  CopyParams params(variant, args);
   if (!pdl) {
-    CUDA_TRY(cudaLaunchKernel(kfn, grid_for(a, ctas), dim3(block_for(variant)), params, smem_for(variant, a), s));
+    CUDA_TRY(cudaLaunchKernel(kfn, grid_for(a, ctas), dim3(block_for(variant)), params.p, smem_for(variant, a), s));
     return MPT_OK;
   }
   cudaLaunchAttribute attr[1];
@@ -194,7 +210,7 @@ mpt_status launch_copy(cudaStream_t s, int variant, const CopyArgs& a, uint32_t 
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  CUDA_TRY(cudaLaunchKernelExC(&cfg, kfn, params));
+  CUDA_TRY(cudaLaunchKernelExC(&cfg, kfn, params.p));
   return MPT_OK;
 }
 
@@ -209,10 +225,10 @@ mpt_status for_each_copy(mpt_ctx_t c, const mpt_plan_s* plan, uint32_t p, const 
     int n = (int)std::min<size_t>(kInlineRanges, ranges.size() - i);
     int variant = base_variant;
     CopyArgs a;
-    mpt_status st = prepare_copy(a, variant, src, dst, ranges.data() + i, n, c->d_status, c->bulk_cfg);
+    uint32_t ctas = spec.ctas;
+    mpt_status st = prepare_copy(c, a, variant, src, dst, ranges.data() + i, n, ctas, plan->dir == MPT_H2D);
     if (st != MPT_OK) return st;
     if (a.ntiles == 0) continue;
-    uint32_t ctas = spec.ctas ? spec.ctas : default_ctas(c, spec.kind, (uint32_t)variant);
     st = emit(variant, a, ctas);
     if (st != MPT_OK) return st;
   }
@@ -468,7 +484,7 @@ mpt_status build_graph(mpt_ctx_t c, const mpt_plan_s* plan, void* dst, const voi
           sa.ready = ready;
           sa.done = ready + nch;
           sa.nchunks = nch;
-          const uint64_t tile = kVecTileVecs * 16;
+          const uint64_t tile = kStageTile;
           sa.tiles_per_chunk = (uint32_t)((cb + tile - 1) / tile);
           sa.status = c->d_status;
           sa.timeout_ns = kDefaultTimeoutNs;
@@ -498,11 +514,12 @@ mpt_status build_graph(mpt_ctx_t c, const mpt_plan_s* plan, void* dst, const voi
             RangeDesc r{ch.offset, slot * cb, ch.bytes, 0, 0};
             int variant = 0;
             CopyArgs a;
-            mpt_status st = prepare_copy(a, variant, src, ds8, &r, 1, c->d_status);
+            uint32_t ctas = spec.ctas;
+            mpt_status st = prepare_copy(c, a, variant, src, ds8, &r, 1, ctas);
             if (st != MPT_OK) return st;
             cudaGraphNode_t h1, h2;
             st = add_copy_node(g->graph, prev_hop2[slot] ? &prev_hop2[slot] : nullptr, prev_hop2[slot] ? 1 : 0, &h1,
-                               variant, a, spec.ctas ? spec.ctas : default_ctas(c, MPT_PATH_SM, 0), info);
+                               variant, a, ctas, info);
             if (st != MPT_OK) return st;
             CUDA_TRY(cudaGraphAddMemcpyNode1D(&h2, g->graph, &h1, 1, d8 + ch.offset, ds8 + slot * cb, ch.bytes,
                                               cudaMemcpyDeviceToHost));
@@ -816,9 +833,10 @@ mpt_status eager(mpt_ctx_t c, const mpt_plan_s* plan, void* dst, const void* src
             RangeDesc r{ch.offset, 0, ch.bytes, 0, 0};
             int variant = 0;
             CopyArgs a;
-            mpt_status st = prepare_copy(a, variant, src, sl, &r, 1, c->d_status);
+            uint32_t ctas = spec.ctas;
+            mpt_status st = prepare_copy(c, a, variant, src, sl, &r, 1, ctas);
             if (st != MPT_OK) return st;
-            st = launch_copy(L.s[0], variant, a, spec.ctas ? spec.ctas : default_ctas(c, MPT_PATH_SM, 0));
+            st = launch_copy(L.s[0], variant, a, ctas);
             if (st != MPT_OK) return st;
           } else {
             CUDA_TRY(cudaMemcpyAsync(sl, s8 + ch.offset, ch.bytes, cudaMemcpyDefault, L.s[0]));
@@ -829,9 +847,10 @@ mpt_status eager(mpt_ctx_t c, const mpt_plan_s* plan, void* dst, const void* src
             RangeDesc r{0, ch.offset, ch.bytes, 0, 0};
             int variant = 0;
             CopyArgs a;
-            mpt_status st = prepare_copy(a, variant, sl, dst, &r, 1, c->d_status);
+            uint32_t ctas = spec.ctas;
+            mpt_status st = prepare_copy(c, a, variant, sl, dst, &r, 1, ctas);
             if (st != MPT_OK) return st;
-            st = launch_copy(L.s[1], variant, a, spec.ctas ? spec.ctas : default_ctas(c, MPT_PATH_SM, 0));
+            st = launch_copy(L.s[1], variant, a, ctas);
             if (st != MPT_OK) return st;
           } else {
             CUDA_TRY(cudaMemcpyAsync(d8 + ch.offset, sl, ch.bytes, cudaMemcpyDefault, L.s[1]));
@@ -1258,10 +1277,9 @@ mpt_status mpt_sm_copy(mpt_ctx_t c, void* dst, const void* src, uint64_t nbytes,
   RangeDesc r{0, 0, nbytes, 0, 0};
   int v = host ? 2 : (variant == MPT_SM_TILE8K ? 3 : (int)variant);
   CopyArgs a;
-  mpt_status st = prepare_copy(a, v, src, dst, &r, 1, c->d_status, c->bulk_cfg);
+  mpt_status st = prepare_copy(c, a, v, src, dst, &r, 1, ctas, ks != kMemDevice);
   if (st != MPT_OK) return st;
-  const uint32_t g = ctas ? ctas : default_ctas(c, host ? MPT_PATH_ZC : MPT_PATH_SM, (uint32_t)v);
-  return launch_copy(static_cast<cudaStream_t>(stream), v, a, g);
+  return launch_copy(static_cast<cudaStream_t>(stream), v, a, ctas);
 }
 
 mpt_status mpt_hash_device(mpt_ctx_t c, const void* ptr, uint64_t nbytes, void* stream, uint64_t* out) {

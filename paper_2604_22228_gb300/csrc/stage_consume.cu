@@ -19,7 +19,7 @@ namespace mpt {
 
 __global__ void __launch_bounds__(kVecThreads) k_stage_consume(StageArgs a) {
   __shared__ int ok;
-  constexpr uint64_t kTile = kVecTileVecs * 16;
+  constexpr uint64_t kTile = kStageTile;
   const uint32_t total = a.nchunks * a.tiles_per_chunk;
   const uint32_t tid = threadIdx.x;
   for (uint32_t t = blockIdx.x; t < total; t += gridDim.x) {
