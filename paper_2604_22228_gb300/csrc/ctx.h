@@ -138,7 +138,9 @@ struct mpt_ctx_s {
   int engines = 0;
   bool pageable = false;              // the GPU reaches pageable host memory (coherent host)
   uint32_t* d_status = nullptr;       // device status word
-  unsigned long long* d_hash = nullptr;
+  unsigned long long* d_hash = nullptr;  // digest accumulator and, behind it, a count of CTAs; zero between calls
+  unsigned long long* h_hash = nullptr;  // page-locked: the digest as the kernel delivers it
+  unsigned long long* h_hash_dev = nullptr;
   uint64_t* d_wait_ns = nullptr;      // device word: wait limit of the staged consumer's flag waits
   mpt::EagerLane lane[MPT_MAX_PATHS];
   cudaEvent_t fork = nullptr;
