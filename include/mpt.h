@@ -8,7 +8,9 @@
  * once as a CUDA graph, cached, and replayed (Sec. 4.2 "CUDA Graph Engine" / "CUDA Graph
  * Cache", Algorithm 1 "LaunchGraph").  On one GPU the paths are:
  *
- *   MPT_PATH_CE  copy-engine DMA, one memcpy per chunk (Algorithm 2 "PeerToPeerCopy");
+ *   MPT_PATH_CE  copy-engine DMA, one memcpy per chunk (Algorithm 2 "PeerToPeerCopy"); over
+ *                the host link chunks that lie side by side move in one memcpy, and from 4 MiB
+ *                the bytes before a source's first 128-byte line in one of their own;
  *   MPT_PATH_SM  a copy kernel driven by the SMs (device-to-device only);
  *   MPT_PATH_HS  a two-hop staged route, hop two of a chunk after its hop one
  *                (Algorithm 2 "StageHostCopy"): device-to-device goes through pinned

@@ -127,6 +127,7 @@ struct mpt_graph_s {
   std::vector<void*> host_allocs, dev_allocs;
   uint64_t src_lo = 0, src_hi = 0, dst_lo = 0, dst_hi = 0;
   bool cached = false;
+  bool ce_split = false;  // host-to-device memcpys begin on lines, the bytes before them apart
   std::list<mpt_graph_s*>::iterator lru_it;
   mpt_plan_s* eager_plan = nullptr;  // set when prepared for direct issue instead of a graph
   std::vector<std::unique_ptr<mpt::HostCopyJob>> host_jobs;  // userData of this graph's host nodes

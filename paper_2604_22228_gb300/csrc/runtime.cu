@@ -126,6 +126,49 @@ std::vector<RangeDesc> path_ranges(const mpt_plan_s* plan, uint32_t p) {
   return out;
 }
 
+// The memcpys of copy-engine path p.  Between device buffers one per chunk.  Over the host link
+// chunks that lie side by side move in one: the link is the bound, and each further memcpy only
+// adds to it (GB300, one message of 464,500 bytes in two chunks of its bucket's plan: 7.0 us on two
+// chains, 6.3 on one, 4.3 as one memcpy; 48 MiB host-to-device in 8 chunks 257 / 255 / 240).
+// `split` (see ce_split_wanted) gives each large one its bytes before a line on their own.
+constexpr uint64_t kHostLine = 128, kSplitMin = 4ull << 20;
+
+struct CePiece {
+  uint64_t offset, bytes;
+};
+
+std::vector<CePiece> ce_pieces(const mpt_plan_s* plan, uint32_t p, const void* src, bool split) {
+  std::vector<CePiece> out;
+  if (plan->dir == MPT_D2D) {
+    for (uint32_t i = plan->first_chunk[p]; i < plan->first_chunk[p + 1]; ++i)
+      out.push_back({plan->chunks[i].offset, plan->chunks[i].bytes});
+    return out;
+  }
+  for (const RangeDesc& r : path_ranges(plan, p)) {
+    uint64_t head = 0;
+    if (split && r.bytes >= kSplitMin) {
+      head = kHostLine - ((reinterpret_cast<uintptr_t>(src) + r.src_off) & (kHostLine - 1));
+      out.push_back({r.src_off, head});
+    }
+    out.push_back({r.src_off + head, r.bytes - head});
+  }
+  return out;
+}
+
+// A copy engine reads host memory from inside a 128-byte line at 176 GB/s instead of 208 (32 MiB:
+// 190.5 us against 161.2; where the destination starts, and device-to-host, does not matter).  The
+// bytes up to the next line as a memcpy of their own cost under 2 us, so from 4 MiB that is the
+// faster way.  A graph keeps the form it was built with when it is retargeted.
+bool ce_split_wanted(const mpt_plan_s* plan, const void* src) {
+  if (plan->dir != MPT_H2D) return false;
+  for (uint32_t p = 0; p < plan->npaths; ++p) {
+    if (plan->paths[p].kind != MPT_PATH_CE) continue;
+    for (const RangeDesc& r : path_ranges(plan, p))
+      if (r.bytes >= kSplitMin && ((reinterpret_cast<uintptr_t>(src) + r.src_off) & (kHostLine - 1))) return true;
+  }
+  return false;
+}
+
 void* kernel_fn(int variant, const CopyArgs& a) {
   return variant == 1 ? const_cast<void*>(bulk_config(a.bulk_cfg).fn) : vec_copy_fn(a, variant == 2);
 }
@@ -308,6 +351,7 @@ mpt_status build_graph(mpt_ctx_t c, const mpt_plan_s* plan, void* dst, const voi
   const double t1 = now_us();
   uint8_t* d8 = static_cast<uint8_t*>(dst);
   const uint8_t* s8 = static_cast<const uint8_t*>(src);
+  g->ce_split = reuse ? reuse->ce_split : ce_split_wanted(plan, src);
 
   for (uint32_t p = 0; p < plan->npaths; ++p) {
     const uint32_t lo = plan->first_chunk[p], hi = plan->first_chunk[p + 1];
@@ -320,14 +364,16 @@ mpt_status build_graph(mpt_ctx_t c, const mpt_plan_s* plan, void* dst, const voi
         // of nodes.  Measured on GB300 (64 MiB in 16 chunks): 32 us as three or four chains,
         // whether graph launches follow each other or not; as 16 independent branches, 34 us
         // alone but 63 us per launch when launches follow each other; as one chain, 50 us.
-        const uint32_t lanes = std::max(1u, std::min(c->ce_lanes, hi - lo));
+        // Over the host link one chain: several only add forks and joins (ce_pieces).
+        const std::vector<CePiece> pieces = ce_pieces(plan, p, src, g->ce_split);
+        const uint32_t lanes = plan->dir == MPT_D2D ? std::max(1u, std::min(c->ce_lanes, hi - lo)) : 1u;
         std::vector<cudaGraphNode_t> tail(lanes, nullptr);
-        for (uint32_t i = lo; i < hi; ++i) {
-          const mpt_chunk& ch = plan->chunks[i];
-          cudaGraphNode_t& prev = tail[(i - lo) % lanes];
+        for (size_t i = 0; i < pieces.size(); ++i) {
+          const CePiece& pc = pieces[i];
+          cudaGraphNode_t& prev = tail[i % lanes];
           cudaGraphNode_t n;
-          CUDA_TRY(cudaGraphAddMemcpyNode1D(&n, g->graph, prev ? &prev : nullptr, prev ? 1 : 0, d8 + ch.offset,
-                                            s8 + ch.offset, ch.bytes, cudaMemcpyDefault));
+          CUDA_TRY(cudaGraphAddMemcpyNode1D(&n, g->graph, prev ? &prev : nullptr, prev ? 1 : 0, d8 + pc.offset,
+                                            s8 + pc.offset, pc.bytes, cudaMemcpyDefault));
           prev = n;
           info.memcpy_nodes++;
         }
@@ -680,15 +726,13 @@ mpt_status eager(mpt_ctx_t c, const mpt_plan_s* plan, void* dst, const void* src
       nonempty++;
       only = p;
     }
-  const bool ce_many = nonempty == 1 && plan->paths[only].kind == MPT_PATH_CE && c->ce_lanes > 1 &&
-                       plan->first_chunk[only + 1] - plan->first_chunk[only] > 1;
+  const bool ce_many = nonempty == 1 && plan->paths[only].kind == MPT_PATH_CE && plan->dir == MPT_D2D &&
+                       c->ce_lanes > 1 && plan->first_chunk[only + 1] - plan->first_chunk[only] > 1;
   if (nonempty == 1 && plan->paths[only].kind != MPT_PATH_HS && !ce_many) {
     if (plan->paths[only].kind == MPT_PATH_CE) {
-      for (uint32_t i = plan->first_chunk[only]; i < plan->first_chunk[only + 1]; ++i) {
-        const mpt_chunk& ch = plan->chunks[i];
-        CUDA_TRY(cudaMemcpyAsync(static_cast<uint8_t*>(dst) + ch.offset, static_cast<const uint8_t*>(src) + ch.offset,
-                                 ch.bytes, cudaMemcpyDefault, user));
-      }
+      for (const CePiece& pc : ce_pieces(plan, only, src, ce_split_wanted(plan, src)))
+        CUDA_TRY(cudaMemcpyAsync(static_cast<uint8_t*>(dst) + pc.offset, static_cast<const uint8_t*>(src) + pc.offset,
+                                 pc.bytes, cudaMemcpyDefault, user));
       return MPT_OK;
     }
     bool pdl = c->pdl;
@@ -743,11 +787,12 @@ mpt_status eager(mpt_ctx_t c, const mpt_plan_s* plan, void* dst, const void* src
     switch (spec.kind) {
       case MPT_PATH_CE: {
         // chunks dealt round robin over the lane's streams, as the graph deals them over chains
-        const uint32_t lanes = std::max(1u, std::min({c->ce_lanes, kLaneStreams, hi - lo}));
+        const std::vector<CePiece> pieces = ce_pieces(plan, p, src, ce_split_wanted(plan, src));
+        const uint32_t lanes = plan->dir == MPT_D2D ? std::max(1u, std::min({c->ce_lanes, kLaneStreams, hi - lo})) : 1u;
         for (uint32_t k = 1; k < lanes; ++k) CUDA_TRY(cudaStreamWaitEvent(L.s[k], c->fork, 0));
-        for (uint32_t i = lo; i < hi; ++i) {
-          const mpt_chunk& ch = plan->chunks[i];
-          CUDA_TRY(cudaMemcpyAsync(d8 + ch.offset, s8 + ch.offset, ch.bytes, cudaMemcpyDefault, L.s[(i - lo) % lanes]));
+        for (size_t i = 0; i < pieces.size(); ++i) {
+          const CePiece& pc = pieces[i];
+          CUDA_TRY(cudaMemcpyAsync(d8 + pc.offset, s8 + pc.offset, pc.bytes, cudaMemcpyDefault, L.s[i % lanes]));
         }
         for (uint32_t k = 1; k < lanes; ++k) {
           CUDA_TRY(cudaEventRecord(L.join[k], L.s[k]));
@@ -1121,7 +1166,8 @@ mpt_status mpt_capture(mpt_ctx_t c, mpt_plan_t plan, void* dst, const void* src,
   if (c->rebind_enabled) {
     for (auto lit = c->lru.rbegin(); lit != c->lru.rend(); ++lit) {
       mpt_graph_s* g = *lit;
-      if (g->refs != 1 || g->key.nbytes != key.nbytes || g->key.dir != key.dir || g->key.plan_hash != key.plan_hash)
+      if (g->refs != 1 || g->key.nbytes != key.nbytes || g->key.dir != key.dir || g->key.plan_hash != key.plan_hash ||
+          g->ce_split != ce_split_wanted(plan, src))
         continue;
       if (rebind(c, g, plan, dst, src) != MPT_OK) break;
       c->cache.erase(g->key);
