@@ -162,7 +162,9 @@ def mpt_prepare(ctx: int, plan: int, dst, src, mode: int = MPT_PREPARE_AUTO) -> 
 
 
 def mpt_launch(graph: int, stream=None) -> None:
-    _check(lib().mpt_launch(graph, _stream(stream)), "mpt_launch")
+    st = (_ffi._lib or lib()).mpt_launch(graph, None if stream is None else getattr(stream, "cuda_stream", stream))
+    if st != MPT_OK:
+        _check(st, "mpt_launch")
 
 
 def mpt_graph_get_info(graph: int) -> dict:

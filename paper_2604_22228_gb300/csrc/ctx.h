@@ -1,5 +1,7 @@
 // Internal context and graph objects (runtime.cu, tuner.cu).
 #pragma once
+#include <cuda.h>
+
 #include <list>
 #include <map>
 #include <memory>
@@ -117,6 +119,23 @@ mpt_model default_model(uint32_t dir, uint32_t mode);
 
 }  // namespace mpt
 
+namespace mpt {
+
+// One operation of a transfer prepared for direct issue on the launching stream: a memcpy, or a
+// copy kernel (fn not null) with its arguments.
+struct DirectOp {
+  CUfunction fn = nullptr;
+  uint32_t grid = 0, block = 0, smem = 0;
+  bool one = false;           // the kernel takes `small`, not `args`
+  CopyArgsT<1> small;
+  CopyArgs args;
+  void* dst = nullptr;
+  const void* src = nullptr;
+  uint64_t bytes = 0;
+};
+
+}  // namespace mpt
+
 struct mpt_graph_s {
   int refs = 0;
   mpt_ctx_t ctx = nullptr;
@@ -130,6 +149,7 @@ struct mpt_graph_s {
   bool ce_split = false;  // host-to-device memcpys begin on lines, the bytes before them apart
   std::list<mpt_graph_s*>::iterator lru_it;
   mpt_plan_s* eager_plan = nullptr;  // set when prepared for direct issue instead of a graph
+  std::vector<mpt::DirectOp> direct;  // and, where that is one path without fork and join, its operations
   std::vector<std::unique_ptr<mpt::HostCopyJob>> host_jobs;  // userData of this graph's host nodes
 };
 

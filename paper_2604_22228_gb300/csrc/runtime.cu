@@ -45,6 +45,18 @@ uint64_t env_u64(const char* name, uint64_t dflt) {
   return (end && *end == 0) ? (uint64_t)x : dflt;
 }
 
+// A function of the driver's interface, looked up by name (null: the driver has none).
+void* driver_entry(const char* name) {
+  void* f = nullptr;
+  cudaDriverEntryPointQueryResult r;
+  if (cudaGetDriverEntryPointByVersion(name, &f, 12000, cudaEnableDefault, &r) != cudaSuccess ||
+      r != cudaDriverEntryPointSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return f;
+}
+
 enum MemKind { kMemDevice, kMemHost, kMemPageable, kMemOther };
 
 // kMemPageable: ordinary (not page-locked) host memory, which the GPU reaches directly
@@ -73,6 +85,7 @@ namespace {
 void graph_destroy_exec(mpt_graph_s* g) {
   delete g->eager_plan;
   g->eager_plan = nullptr;
+  g->direct.clear();
   // A launch still in flight may not have run its host nodes yet: their jobs must outlive it.
   if (!g->host_jobs.empty()) cudaDeviceSynchronize();
   g->host_jobs.clear();
@@ -716,11 +729,10 @@ mpt_status grow_dev(EagerLane& L, uint64_t bytes) {
   return MPT_OK;
 }
 
-mpt_status eager(mpt_ctx_t c, const mpt_plan_s* plan, void* dst, const void* src, cudaStream_t user) {
-  if (plan->nbytes == 0) return MPT_OK;
-  // One copy-engine or kernel path needs no fork and join: issue it on the caller's
-  // stream directly (the cheapest launch for short messages).
-  uint32_t nonempty = 0, only = 0;
+// One copy-engine or kernel path needs no fork and join: it is issued on the caller's stream
+// directly (the cheapest launch for short messages).  Stores that path in `only`.
+bool one_direct_path(mpt_ctx_t c, const mpt_plan_s* plan, uint32_t& only) {
+  uint32_t nonempty = 0;
   for (uint32_t p = 0; p < plan->npaths; ++p)
     if (plan->first_chunk[p + 1] > plan->first_chunk[p]) {
       nonempty++;
@@ -728,22 +740,90 @@ mpt_status eager(mpt_ctx_t c, const mpt_plan_s* plan, void* dst, const void* src
     }
   const bool ce_many = nonempty == 1 && plan->paths[only].kind == MPT_PATH_CE && plan->dir == MPT_D2D &&
                        c->ce_lanes > 1 && plan->first_chunk[only + 1] - plan->first_chunk[only] > 1;
-  if (nonempty == 1 && plan->paths[only].kind != MPT_PATH_HS && !ce_many) {
+  return nonempty == 1 && plan->paths[only].kind != MPT_PATH_HS && !ce_many;
+}
+
+// Programmatic dependent launch is not used inside a stream capture.
+bool pdl_allowed(mpt_ctx_t c, cudaStream_t user) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (!c->pdl) return false;
+  if (cudaStreamIsCapturing(user, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return cap == cudaStreamCaptureStatusNone;
+}
+
+// The operations of a plan's one direct path, made once for a handle's many launches: a launch
+// then costs its driver call and little else (64 messages of 8 B to 64 KiB a pass: 146 us with the
+// path's ranges and arguments built at every launch, 119 now).
+mpt_status prepare_direct(mpt_ctx_t c, const mpt_plan_s* plan, void* dst, const void* src,
+                          std::vector<DirectOp>& ops) {
+  ops.clear();
+  uint32_t only = 0;
+  if (plan->nbytes == 0 || !one_direct_path(c, plan, only)) return MPT_OK;
+  if (plan->paths[only].kind == MPT_PATH_CE) {
+    for (const CePiece& pc : ce_pieces(plan, only, src, ce_split_wanted(plan, src))) {
+      ops.emplace_back();
+      ops.back().dst = static_cast<uint8_t*>(dst) + pc.offset;
+      ops.back().src = static_cast<const uint8_t*>(src) + pc.offset;
+      ops.back().bytes = pc.bytes;
+    }
+    return MPT_OK;
+  }
+  return for_each_copy(c, plan, only, src, dst, [&](int variant, const CopyArgs& a, uint32_t ctas) -> mpt_status {
+    ops.emplace_back();
+    DirectOp& op = ops.back();
+    op.args = a;
+    const CopyParams params(variant, op.args);
+    op.one = params.p[0] != &op.args;
+    if (op.one) op.small = params.one;
+    op.grid = grid_for(a, ctas).x;
+    op.block = block_for(variant);
+    op.smem = (uint32_t)smem_for(variant, a);
+    CUDA_TRY(cudaGetFuncBySymbol(reinterpret_cast<cudaFunction_t*>(&op.fn), kernel_fn(variant, a)));
+    return MPT_OK;
+  });
+}
+
+mpt_status issue_direct(mpt_ctx_t c, std::vector<DirectOp>& ops, cudaStream_t user) {
+  static const auto launch_kernel = reinterpret_cast<CUresult (*)(const CUlaunchConfig*, CUfunction, void**, void**)>(
+      driver_entry("cuLaunchKernelEx"));
+  if (!launch_kernel) return fail(MPT_ECUDA, "mpt_launch: the driver has no cuLaunchKernelEx");
+  for (DirectOp& op : ops) {
+    if (!op.fn) {
+      CUDA_TRY(cudaMemcpyAsync(op.dst, op.src, op.bytes, cudaMemcpyDefault, user));
+      continue;
+    }
+    CUlaunchAttribute attr[1];
+    attr[0].id = CU_LAUNCH_ATTRIBUTE_PROGRAMMATIC_STREAM_SERIALIZATION;
+    attr[0].value.programmaticStreamSerializationAllowed = 1;
+    CUlaunchConfig cfg{};
+    cfg.gridDimX = op.grid;
+    cfg.gridDimY = cfg.gridDimZ = cfg.blockDimY = cfg.blockDimZ = 1;
+    cfg.blockDimX = op.block;
+    cfg.sharedMemBytes = op.smem;
+    cfg.hStream = user;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl_allowed(c, user) ? 1 : 0;
+    void* params[] = {op.one ? static_cast<void*>(&op.small) : static_cast<void*>(&op.args)};
+    const CUresult e = launch_kernel(&cfg, op.fn, params, nullptr);
+    if (e != CUDA_SUCCESS) return fail(MPT_ECUDA, "mpt_launch: copy kernel launch: driver error %d", (int)e);
+  }
+  return MPT_OK;
+}
+
+mpt_status eager(mpt_ctx_t c, const mpt_plan_s* plan, void* dst, const void* src, cudaStream_t user) {
+  if (plan->nbytes == 0) return MPT_OK;
+  uint32_t only = 0;
+  if (one_direct_path(c, plan, only)) {
     if (plan->paths[only].kind == MPT_PATH_CE) {
       for (const CePiece& pc : ce_pieces(plan, only, src, ce_split_wanted(plan, src)))
         CUDA_TRY(cudaMemcpyAsync(static_cast<uint8_t*>(dst) + pc.offset, static_cast<const uint8_t*>(src) + pc.offset,
                                  pc.bytes, cudaMemcpyDefault, user));
       return MPT_OK;
     }
-    bool pdl = c->pdl;
-    if (pdl) {
-      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-      if (cudaStreamIsCapturing(user, &cap) != cudaSuccess) {
-        cudaGetLastError();
-        pdl = false;
-      }
-      if (cap != cudaStreamCaptureStatusNone) pdl = false;
-    }
+    const bool pdl = pdl_allowed(c, user);
     return for_each_copy(c, plan, only, src, dst, [&](int variant, const CopyArgs& a, uint32_t ctas) {
       return launch_copy(user, variant, a, ctas, pdl);
     });
@@ -1224,6 +1304,11 @@ mpt_status mpt_prepare(mpt_ctx_t c, mpt_plan_t plan, void* dst, const void* src,
   g->ctx = c;
   g->key = GraphKey{(uint64_t)(uintptr_t)src, (uint64_t)(uintptr_t)dst, plan->nbytes, plan->dir, plan->hash};
   set_range(g, plan->nbytes, dst, src);
+  mpt_status st = prepare_direct(c, plan, dst, src, g->direct);
+  if (st != MPT_OK) {
+    delete g;
+    return st;
+  }
   g->eager_plan = new mpt_plan_s(*plan);
   g->info.mode = 1;
   g->refs = 1;
@@ -1237,6 +1322,7 @@ mpt_status mpt_launch(mpt_graph_t g, void* stream) {
   if (!g->ctx) return fail(MPT_EINVAL, "mpt_launch: the graph's context was destroyed");
   if (g->eager_plan) {  // prepared for direct issue (mpt_prepare chose eager)
     CUDA_TRY(cudaSetDevice(g->ctx->device));
+    if (!g->direct.empty()) return issue_direct(g->ctx, g->direct, static_cast<cudaStream_t>(stream));
     return eager(g->ctx, g->eager_plan, reinterpret_cast<void*>(g->key.dst), reinterpret_cast<const void*>(g->key.src),
                  static_cast<cudaStream_t>(stream));
   }
@@ -1269,6 +1355,7 @@ mpt_status mpt_graph_rebind(mpt_graph_t g, mpt_plan_t plan, void* dst, const voi
       return fail(MPT_EAGAIN, "mpt_graph_rebind: another cached graph already serves these addresses");
   }
   mpt_status st = rebind(c, g, plan, dst, src);
+  if (st == MPT_OK && g->eager_plan) st = prepare_direct(c, plan, dst, src, g->direct);
   if (st != MPT_OK) return st;
   if (g->cached) {
     c->cache.erase(g->key);

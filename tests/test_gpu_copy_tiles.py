@@ -75,3 +75,38 @@ def test_many_ranges_in_one_launch(ctx, offsets):
     assert np.array_equal(dst.numpy(), T.copy(data)) and dst.guards_intact()
     mpt.mpt_graph_release(h)
     mpt.mpt_plan_destroy(plan)
+
+
+@pytest.mark.parametrize("paths", [[(mpt.MPT_PATH_SM, 65536, 64 * KiB)], [(mpt.MPT_PATH_CE, 65536, 1024 * KiB)],
+                                   [(mpt.MPT_PATH_SM, 65536, 64 * KiB, 0, mpt.MPT_SM_BULK)],
+                                   [(mpt.MPT_PATH_CE, 32768, 64 * KiB), (mpt.MPT_PATH_SM, 32768, 64 * KiB)]],
+                         ids=["sm", "ce", "bulk", "split"])
+def test_direct_issue_handle_retargeted(ctx, paths):
+    """A handle prepared for direct issue moves between its newest addresses, in a stream capture
+    as well."""
+    import torch
+    n = 300 * KiB + 9
+    pairs = []
+    for so, do in ((0, 0), (16, 0), (3, 40)):
+        src, dst = Buf(n, "dev", so), Buf(n, "dev", do)
+        data = seeded("u8", 0xD1 + so, n)
+        src.fill(data)
+        pairs.append((src, dst, data))
+    plan = mpt.mpt_plan(ctx, n, mpt.MPT_D2D, paths)
+    h = mpt.mpt_prepare(ctx, plan, pairs[0][1].ptr, pairs[0][0].ptr, mpt.MPT_PREPARE_EAGER)
+    s = torch.cuda.Stream()
+    for i, (src, dst, data) in enumerate(pairs):
+        if i:
+            mpt.mpt_graph_rebind(h, plan, dst.ptr, src.ptr)
+        mpt.mpt_launch(h, s)
+        assert np.array_equal(dst.numpy(), T.copy(data)) and dst.guards_intact(), i
+    src, dst, data = pairs[2]
+    dst.view.zero_()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s, capture_error_mode="thread_local"):
+        mpt.mpt_launch(h, s)
+    g.replay()
+    assert np.array_equal(dst.numpy(), T.copy(data))
+    mpt.mpt_graph_release(h)
+    mpt.mpt_plan_destroy(plan)
