@@ -645,7 +645,8 @@ MPT_API mpt_status mpt_serve_stop(mpt_server_t server);
  * x cols fp32 row-major device arrays, rows 0 and rows+1 the halos.  Interior points:
  * out[r][c] = ((in[r-1][c] + in[r+1][c]) + (in[r][c-1] + in[r][c+1])) * 0.25, each operation
  * rounded to fp32 in that order; columns 0 and cols-1 copied; out's halo rows untouched.
- * Asynchronous on `stream` (legal inside a stream capture).  Errors: EINVAL. */
+ * Asynchronous on `stream` (legal inside a stream capture; outside one the launch overlaps the
+ * end of the kernel before it on `stream`, as direct copies do).  Errors: EINVAL. */
 MPT_API mpt_status mpt_demo_jacobi_step(const float* in, float* out, uint32_t rows, uint64_t cols, void* stream);
 
 /* ---- failure detection self-test ---------------------------------------------------- */

@@ -13,6 +13,7 @@
 // `out` are not written.
 #include <algorithm>
 
+#include "copy_device.cuh"
 #include "internal.h"
 
 namespace mpt {
@@ -52,6 +53,7 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_v4(const float* __restrict_
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t nq = cols / 4;
   const uint64_t q = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_enter();
   if (q - lane >= nq) return;  // a warp past the row's end
   const bool active = q < nq;
   const uint64_t c0 = 4 * (active ? q : nq - 1);  // idle lanes shadow the last quad (shuffles need them)
@@ -97,6 +99,7 @@ __global__ void __launch_bounds__(kThreads) k_jacobi(const float* __restrict__ i
                                                      uint32_t rows, uint64_t cols) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t w0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x - lane) * kG;  // the warp's first column
+  pdl_enter();
   if (w0 >= cols) return;
   const uint64_t c0 = w0 + lane;
   const uint64_t w1 = w0 + 32 * kG;  // one past its last column
@@ -139,17 +142,33 @@ __global__ void __launch_bounds__(kThreads) k_jacobi(const float* __restrict__ i
   }
 }
 
-// Blocks of 8 warps: across a row where it is wide enough, else over strips of rows too.
+// Blocks of 8 warps: across a row where it is wide enough, else over strips of rows too.  Outside a
+// stream capture the launch overlaps the end of the kernel ahead, as the copy kernels' does; each
+// waits for that kernel before it touches memory (a ring of four 1024 x 4096 subdomains, two
+// iterations with their halo copies: 91.7 us without, 78.3 with; 8 x 4 Mi 460 and 438).
 template <typename Kernel>
-void launch(Kernel k, uint32_t warp_cols, uint32_t strip, const float* in, float* out, uint32_t rows, uint64_t cols,
-            cudaStream_t s) {
+cudaError_t launch(Kernel k, uint32_t warp_cols, uint32_t strip, const float* in, float* out, uint32_t rows,
+                   uint64_t cols, cudaStream_t s) {
   const uint64_t nxw = (cols + warp_cols - 1) / warp_cols;  // warps across a row
   uint32_t bx = 1;
   while (bx < kThreads / 32 && bx < nxw) bx <<= 1;
   const uint32_t by = kThreads / 32 / bx;
   const uint32_t nstrips = rows / strip + (rows % strip != 0);
-  const dim3 grid((uint32_t)((nxw + bx - 1) / bx), std::min<uint32_t>((nstrips + by - 1) / by, 65535u));
-  k<<<grid, dim3(32 * bx, by), 0, s>>>(in, out, rows, cols);
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    cap = cudaStreamCaptureStatusActive;
+  }
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((uint32_t)((nxw + bx - 1) / bx), std::min<uint32_t>((nstrips + by - 1) / by, 65535u));
+  cfg.blockDim = dim3(32 * bx, by);
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, k, in, out, rows, cols);
 }
 
 }  // namespace
@@ -165,17 +184,17 @@ extern "C" MPT_API mpt_status mpt_demo_jacobi_step(const float* in, float* out, 
   if (blocks > 0x7fffffffull) return mpt::fail(MPT_EINVAL, "mpt_demo_jacobi_step: %llu columns", (unsigned long long)cols);
   using namespace mpt;
   const uint64_t points = (uint64_t)rows * cols;
+  cudaError_t e;
   if (vec) {
-    if (rows == 1) launch(k_jacobi_v4<1>, 128, 1, in, out, rows, cols, s);
-    else if (rows == 2 || points < kSmallGrid) launch(k_jacobi_v4<2>, 128, 2, in, out, rows, cols, s);
-    else if (rows <= 4 || points < kLargeGrid) launch(k_jacobi_v4<4>, 128, 4, in, out, rows, cols, s);
-    else launch(k_jacobi_v4<8>, 128, 8, in, out, rows, cols, s);
+    if (rows == 1) e = launch(k_jacobi_v4<1>, 128, 1, in, out, rows, cols, s);
+    else if (rows == 2 || points < kSmallGrid) e = launch(k_jacobi_v4<2>, 128, 2, in, out, rows, cols, s);
+    else if (rows <= 4 || points < kLargeGrid) e = launch(k_jacobi_v4<4>, 128, 4, in, out, rows, cols, s);
+    else e = launch(k_jacobi_v4<8>, 128, 8, in, out, rows, cols, s);
   } else {
-    if (points < kTinyGrid) launch(k_jacobi<1, 1>, 32, 1, in, out, rows, cols, s);
-    else if (rows <= 3 || points < kSmallGrid) launch(k_jacobi<2, 4>, 128, 2, in, out, rows, cols, s);
-    else launch(k_jacobi<4, 4>, 128, 4, in, out, rows, cols, s);
+    if (points < kTinyGrid) e = launch(k_jacobi<1, 1>, 32, 1, in, out, rows, cols, s);
+    else if (rows <= 3 || points < kSmallGrid) e = launch(k_jacobi<2, 4>, 128, 2, in, out, rows, cols, s);
+    else e = launch(k_jacobi<4, 4>, 128, 4, in, out, rows, cols, s);
   }
-  const cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return mpt::fail(MPT_ECUDA, "mpt_demo_jacobi_step: %s", cudaGetErrorString(e));
+  if (e != cudaSuccess) return fail(MPT_ECUDA, "mpt_demo_jacobi_step: %s", cudaGetErrorString(e));
   return MPT_OK;
 }

@@ -31,3 +31,39 @@ def test_sweep_at_strip_edges(rows, cols, offset):
     assert np.array_equal(got[1:rows + 1], J.step(grid)[1:rows + 1])
     assert (got[0] == 7.0).all() and (got[rows + 1] == 7.0).all()  # halo rows are not written
     assert (buf_out[:offset].cpu().numpy() == 7.0).all() and (buf_out[offset + n:].cpu().numpy() == 7.0).all()
+
+
+@pytest.mark.parametrize("rows,cols", [(3, 64), (40, 513), (600, 2048)])
+def test_chain_of_sweeps_and_copies(rows, cols):
+    """Back-to-back sweeps between two buffers, each reading what the one before wrote, with a
+    directly issued copy of the grid after every fourth: launches overlap, memory does not."""
+    import torch
+    n = (rows + 2) * cols
+    grid = payload.fill("f32", 0x5EED000C + rows, n * 4).view(np.float32).reshape(rows + 2, cols)
+    want = grid.copy()
+    a, b = torch.from_numpy(grid.copy()).cuda(), torch.from_numpy(grid.copy()).cuda()
+    c = torch.zeros_like(a)
+    ctx = mpt.mpt_ctx_create(0)
+    plan = mpt.mpt_plan(ctx, n * 4, mpt.MPT_D2D, [(mpt.MPT_PATH_SM, 65536, n * 4 // 16 * 16)])
+    out = [mpt.mpt_prepare(ctx, plan, c, x, mpt.MPT_PREPARE_EAGER) for x in (a, b)]
+    back = [mpt.mpt_prepare(ctx, plan, x, c, mpt.MPT_PREPARE_EAGER) for x in (a, b)]
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for it in range(40):
+        mpt.mpt_demo_jacobi_step(a, b, rows, cols, s)
+        new = want.copy()
+        new[1:rows + 1] = J.step(want)[1:rows + 1]
+        want = new
+        a, b = b, a
+        out.reverse()
+        back.reverse()
+        if it % 4 == 3:  # a -> c -> b: the next sweep overwrites b from a
+            mpt.mpt_launch(out[0], s)
+            mpt.mpt_launch(back[1], s)
+    s.synchronize()
+    assert np.array_equal(a.cpu().numpy(), want)
+    assert np.array_equal(c.cpu().numpy(), want) and np.array_equal(b.cpu().numpy(), want)
+    for h in out + back:
+        mpt.mpt_graph_release(h)
+    mpt.mpt_plan_destroy(plan)
+    mpt.mpt_ctx_destroy(ctx)
