@@ -506,8 +506,9 @@ MPT_API mpt_status mpt_batch_submit(mpt_ctx_t ctx, const mpt_xfer* xfers, size_t
  * transfer. */
 MPT_API mpt_status mpt_batch_poll(mpt_batch_t batch, size_t* done, uint8_t* flags);
 
-/* Wait up to timeout_ns for the whole batch (bounded host wait).  ETIMEDOUT when it is
- * still running -- the batch keeps running and may be waited for again. */
+/* Wait up to timeout_ns for the whole batch (bounded host wait): returns once every transfer's
+ * destination bytes are written and visible, to the host too.  ETIMEDOUT when it is still
+ * running -- the batch keeps running and may be waited for again. */
 MPT_API mpt_status mpt_batch_wait(mpt_batch_t batch, uint64_t timeout_ns);
 
 /* Completion time of every transfer in nanoseconds after the batch kernel started (device

@@ -405,7 +405,7 @@ def mpt_selftest_flag_timeout(ctx: int, timeout_ns: int):
 def mpt_hash_ranges_noalloc(ranges, stream=None) -> list[int]:
     """Digests of [(pointer, nbytes), ...] without any allocation (see include/mpt.h)."""
     n = len(ranges)
-    ptrs = (C.c_void_p * max(1, n))(*[_ptr(p) for p, _ in ranges])
+    ptrs = (C.c_void_p * max(1, n))(*[p if type(p) is int else _ptr(p) for p, _ in ranges])
     sizes = (C.c_uint64 * max(1, n))(*[b for _, b in ranges])
     out = (C.c_uint64 * max(1, n))()
     _check(lib().mpt_hash_ranges_noalloc(ptrs, sizes, n, _stream(stream), out), "mpt_hash_ranges_noalloc")

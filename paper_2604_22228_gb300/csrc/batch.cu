@@ -19,6 +19,7 @@
 // it ends, so no reset node runs between replays: a one-request batch costs one small copy
 // and one kernel.
 #include <algorithm>
+#include <atomic>
 #include <iterator>
 #include <chrono>
 #include <cmath>
@@ -407,11 +408,17 @@ mpt_status slot_init(mpt_ctx_t c, BatchSlot& s, uint32_t max_xfers, uint32_t cta
   return MPT_OK;
 }
 
-// Classify [p, p+n) against registered arenas (fast path) or the CUDA runtime.
-int range_kind(mpt_ctx_t c, const void* p, uint64_t n) {
+// Classify [p, p+n) against registered arenas (fast path; `hint`, the arena that held the range
+// before it, first) or the CUDA runtime.
+int range_kind(mpt_ctx_t c, const void* p, uint64_t n, size_t& hint) {
   const uint64_t a = (uint64_t)(uintptr_t)p;
-  for (const Arena& r : c->arenas)
-    if (a >= r.base && a + n <= r.base + r.bytes && a + n >= a) return r.kind;
+  const auto holds = [&](const Arena& r) { return a >= r.base && a + n <= r.base + r.bytes && a + n >= a; };
+  if (hint < c->arenas.size() && holds(c->arenas[hint])) return c->arenas[hint].kind;
+  for (size_t i = 0; i < c->arenas.size(); ++i)
+    if (holds(c->arenas[i])) {
+      hint = i;
+      return c->arenas[i].kind;
+    }
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
@@ -468,12 +475,14 @@ void batch_teardown(mpt_ctx_t c) {
   c->each_ev.clear();
 }
 
-mpt_status batch_check_xfer(mpt_ctx_t c, const mpt_xfer& x, int* src_kind, int* dst_kind) {
+mpt_status batch_check_xfer(mpt_ctx_t c, const mpt_xfer& x, int* src_kind, int* dst_kind, ArenaHints* hints) {
+  ArenaHints none;
+  if (!hints) hints = &none;
   *src_kind = *dst_kind = -1;
   if (x.dir > MPT_D2H) return fail(MPT_EINVAL, "transfer has direction %u", x.dir);
   if (x.bytes == 0) return MPT_OK;
   if (!x.src || !x.dst) return fail(MPT_EINVAL, "transfer has a NULL pointer");
-  const int ks = range_kind(c, x.src, x.bytes), kd = range_kind(c, x.dst, x.bytes);
+  const int ks = range_kind(c, x.src, x.bytes, hints->src[x.dir]), kd = range_kind(c, x.dst, x.bytes, hints->dst[x.dir]);
   const int want_s = x.dir == MPT_H2D ? 1 : 0, want_d = x.dir == MPT_D2H ? 1 : 0;
   if ((ks == 2 ? 1 : ks) != want_s || (kd == 2 ? 1 : kd) != want_d)
     return fail(MPT_EINVAL, "transfer pointers do not match direction %u", x.dir);
@@ -497,6 +506,8 @@ uint64_t mpt::batch_cta_spread_ns(mpt_batch_t b) {
   const uint64_t first = t[0], last = t[1];
   return last >= first ? last - first : 0;
 }
+
+bool mpt::batch_finished(mpt_batch_t b) { return cudaEventQuery(b->ctx->slots[b->slot].done_ev) == cudaSuccess; }
 
 float mpt::batch_gpu_ms(mpt_batch_t b) {
   const mpt::BatchSlot& s = b->ctx->slots[b->slot];
@@ -649,35 +660,67 @@ mpt_status mpt_batch_submit(mpt_ctx_t c, const mpt_xfer* xfers, size_t n, void* 
   if (st != MPT_OK) return st;
   if (n == 0 || n > c->slots[0].max_xfers)
     return fail(MPT_EINVAL, "mpt_batch_submit: %zu transfers (1..%u per batch)", n, c->slots[0].max_xfers);
-  uint32_t si = 0;
-  while (si < c->slots.size() && c->slots[si].held) ++si;
+  // a free slot whose previous batch has left the GPU, else any free one
+  uint32_t si = (uint32_t)c->slots.size();
+  for (uint32_t i = 0; i < c->slots.size(); ++i) {
+    if (c->slots[i].held) continue;
+    if (si == c->slots.size()) si = i;
+    if (cudaEventQuery(c->slots[i].done_ev) == cudaSuccess) {
+      si = i;
+      break;
+    }
+  }
   if (si == c->slots.size()) return fail(MPT_EAGAIN, "mpt_batch_submit: every batch slot is held");
   BatchSlot& s = c->slots[si];
   // validate: direction, memory kinds, and non-overlapping destinations (Sec. 4.5: each
-  // transfer owns its destination region)
-  // scratch owned by the context (one thread per context): no allocation per batch
-  std::vector<std::pair<uint64_t, uint64_t>>& spans = c->batch_spans;
-  spans.clear();
+  // transfer owns its destination region).  Scratch owned by the context (one thread per
+  // context): no allocation per batch.  Destinations are kept apart by memory kind, as ranges of
+  // different kinds cannot overlap: a batch packed in order is then found in order, and sources
+  // outside every destination's span are settled by one comparison (4096 transfers: 130 us of
+  // host time for a sort and 4096 searches before, 85 now).
   std::vector<uint32_t>& dma_cand = c->batch_cand;  // entries large enough for a copy-engine lane
   dma_cand.clear();
+  bool in_order[2] = {true, true};
+  for (auto& spans : c->batch_spans) spans.clear();
+  ArenaHints hints;
+  // two classes of tiles, link (a host side) and device; one class when the split is off
+  const auto cls_of = [&](const mpt_xfer& x) { return (c->batch_split && x.dir == MPT_D2D) ? 1 : 0; };
+  bool any_shift = false;
+  uint64_t cls_bytes[2] = {0, 0};
+  uint32_t cls_n[2] = {0, 0};
+  const auto count = [&](const mpt_xfer& x) {
+    any_shift |= (((uintptr_t)x.src ^ (uintptr_t)x.dst) & 15) != 0 && x.bytes >= 16;
+    cls_bytes[cls_of(x)] += x.bytes;
+    cls_n[cls_of(x)]++;
+  };
   for (size_t i = 0; i < n; ++i) {
     const mpt_xfer& x = xfers[i];
     int ks, kd;
-    if (batch_check_xfer(c, x, &ks, &kd) != MPT_OK)
+    if (batch_check_xfer(c, x, &ks, &kd, &hints) != MPT_OK)
       return fail(MPT_EINVAL, "mpt_batch_submit: transfer %zu: %s", i, mpt_last_error());
+    count(x);
     if (x.bytes == 0) continue;
-    spans.emplace_back((uint64_t)(uintptr_t)x.dst, (uint64_t)(uintptr_t)x.dst + x.bytes);
+    auto& spans = c->batch_spans[kd != 0];
+    const uint64_t lo = (uint64_t)(uintptr_t)x.dst;
+    if (!spans.empty() && lo < spans.back().second) in_order[kd != 0] = false;
+    spans.emplace_back(lo, lo + x.bytes);
     if (s.dma_lanes && x.bytes >= c->batch_dma_min && ks != 2 && kd != 2) dma_cand.push_back((uint32_t)i);
   }
-  std::sort(spans.begin(), spans.end());
-  for (size_t i = 1; i < spans.size(); ++i)
-    if (spans[i].first < spans[i - 1].second)
-      return fail(MPT_EINVAL, "mpt_batch_submit: destination regions overlap");
+  for (int k = 0; k < 2; ++k) {
+    if (in_order[k]) continue;  // each begins at or after the end of the one before it
+    auto& spans = c->batch_spans[k];
+    std::sort(spans.begin(), spans.end());
+    for (size_t i = 1; i < spans.size(); ++i)
+      if (spans[i].first < spans[i - 1].second)
+        return fail(MPT_EINVAL, "mpt_batch_submit: destination regions overlap");
+  }
   // no source may overlap a destination: the batch's transfers run at the same time
   for (size_t i = 0; i < n; ++i) {
     const mpt_xfer& x = xfers[i];
-    if (x.bytes == 0) continue;
+    const auto& spans = c->batch_spans[x.dir == MPT_H2D];
+    if (x.bytes == 0 || spans.empty()) continue;
     const uint64_t a = (uint64_t)(uintptr_t)x.src, b = a + x.bytes;
+    if (a >= spans.back().second || b <= spans.front().first) continue;
     // spans are sorted and disjoint: only the last one starting at or before a, and the
     // first one starting after a, can reach into [a, b)
     auto it = std::upper_bound(spans.begin(), spans.end(), std::pair<uint64_t, uint64_t>(a, UINT64_MAX));
@@ -691,10 +734,11 @@ mpt_status mpt_batch_submit(mpt_ctx_t c, const mpt_xfer* xfers, size_t n, void* 
   // DMA lanes: largest eligible entries first, each to the least-loaded lane of its
   // direction with a free item (longest-processing-time order); the rest stay with the kernel
   const uint32_t ndma = kDmaDirs * s.dma_lanes * s.dma_items;
-  std::vector<uint8_t>& to_dma = c->batch_to_dma;
-  to_dma.assign(n, 0);
+  std::vector<uint8_t>& to_dma = c->batch_to_dma;  // empty: none
+  to_dma.clear();
   for (uint32_t k = 0; k < ndma; ++k) s.h_dma_map[k] = ~0u;
   if (!dma_cand.empty()) {
+    to_dma.assign(n, 0);
     std::sort(dma_cand.begin(), dma_cand.end(),
               [&](uint32_t a, uint32_t b) { return xfers[a].bytes > xfers[b].bytes || (xfers[a].bytes == xfers[b].bytes && a < b); });
     std::vector<uint64_t> load(kDmaDirs * s.dma_lanes, 0);
@@ -713,17 +757,12 @@ mpt_status mpt_batch_submit(mpt_ctx_t c, const mpt_xfer* xfers, size_t n, void* 
       to_dma[i] = 1;
     }
   }
-  // two classes of tiles, link (a host side) and device; one class when the split is off
-  const auto cls_of = [&](const mpt_xfer& x) { return (c->batch_split && x.dir == MPT_D2D) ? 1 : 0; };
-  bool any_shift = false;
-  uint64_t cls_bytes[2] = {0, 0};
-  uint32_t cls_n[2] = {0, 0};
-  for (size_t i = 0; i < n; ++i) {
-    if (to_dma[i]) continue;
-    const mpt_xfer& x = xfers[i];
-    any_shift |= (((uintptr_t)x.src ^ (uintptr_t)x.dst) & 15) != 0 && x.bytes >= 16;
-    cls_bytes[cls_of(x)] += x.bytes;
-    cls_n[cls_of(x)]++;
+  if (!to_dma.empty()) {  // the kernel's share is what the lanes leave
+    any_shift = false;
+    cls_bytes[0] = cls_bytes[1] = 0;
+    cls_n[0] = cls_n[1] = 0;
+    for (size_t i = 0; i < n; ++i)
+      if (!to_dma[i]) count(xfers[i]);
   }
   const int gi = any_shift ? 1 : 0;
   const uint32_t ctas = grid_ctas(c);
@@ -746,12 +785,13 @@ mpt_status mpt_batch_submit(mpt_ctx_t c, const mpt_xfer* xfers, size_t n, void* 
   uint64_t tiles[2] = {0, 0};
   uint32_t at[2] = {0, cls_n[0]};
   for (size_t i = 0; i < n; ++i) {
-    if (to_dma[i]) continue;
+    if (!to_dma.empty() && to_dma[i]) continue;
     const mpt_xfer& x = xfers[i];
     const int k = cls_of(x);
     const uint32_t fl = (x.dir == MPT_D2H ? kDescHostDst : 0u) | (x.dir != MPT_D2D ? kDescHostSide : 0u);
     const uint64_t lead = (uintptr_t)(x.dir == MPT_H2D ? x.src : x.dst) & (kLine - 1);
-    const uint64_t t = std::max<uint64_t>(1, (x.bytes + lead + tile[k] - 1) / tile[k]);
+    // (one tile, the usual case of a short transfer, without the division)
+    const uint64_t t = x.bytes + lead <= tile[k] ? 1 : (x.bytes + lead + tile[k] - 1) / tile[k];
     first[at[k]] = (uint32_t)tiles[k];
     d[at[k]++] = BatchDesc{(uint64_t)(uintptr_t)x.src, (uint64_t)(uintptr_t)x.dst, x.bytes, (uint32_t)tiles[k],
                            (uint32_t)t, fl, (uint32_t)i};
@@ -815,6 +855,7 @@ mpt_status mpt_batch_poll(mpt_batch_t b, size_t* done, uint8_t* flags) {
     k += fin;
     if (flags) flags[i] = fin ? 1 : 0;
   }
+  std::atomic_thread_fence(std::memory_order_acquire);
   *done = k;
   return MPT_OK;
 }
@@ -823,13 +864,23 @@ mpt_status mpt_batch_wait(mpt_batch_t b, uint64_t timeout_ns) {
   if (!b) return fail(MPT_EINVAL, "mpt_batch_wait: NULL batch");
   const BatchSlot& s = b->ctx->slots[b->slot];
   const uint64_t t0 = host_ns();
-  while (true) {
+  // The batch is done when every transfer's flag is up: the kernel raises a flag behind its
+  // transfer's bytes, and sees to its counters after the last.  The completion event, some 4 us
+  // later (a lone 64 KiB transfer from submission: 18.9 us by the event, 14.4 by its flag), is
+  // asked now and then for errors.
+  volatile const uint32_t* f = s.h_flags;
+  size_t lo = 0;
+  for (uint32_t turn = 0;; ++turn) {
+    while (lo < b->n && f[lo] == b->epoch) ++lo;
+    if (lo == b->n) break;
+    if (turn % 64) continue;
     const cudaError_t e = cudaEventQuery(s.done_ev);
     if (e == cudaSuccess) break;
     if (e != cudaErrorNotReady) return fail(MPT_ECUDA, "mpt_batch_wait: %s", cudaGetErrorString(e));
     if (host_ns() - t0 >= timeout_ns) return fail(MPT_ETIMEDOUT, "mpt_batch_wait: batch still running");
     std::this_thread::yield();
   }
+  std::atomic_thread_fence(std::memory_order_acquire);  // destinations in host memory are read after the flags
   return MPT_OK;
 }
 
@@ -875,6 +926,7 @@ mpt_status mpt_batch_watch(mpt_batch_t b, uint64_t t0_ns, uint64_t* out_ns, uint
     if (e != cudaErrorNotReady) return fail(MPT_ECUDA, "mpt_batch_watch: %s", cudaGetErrorString(e));
     if (now - start >= timeout_ns) return fail(MPT_ETIMEDOUT, "mpt_batch_watch: batch still running");
   }
+  std::atomic_thread_fence(std::memory_order_acquire);
   return MPT_OK;
 }
 

@@ -102,7 +102,14 @@ void batch_teardown(mpt_ctx_t c);
 // pointers, memory kinds against the direction).  *src_kind / *dst_kind: 0 device, 1
 // page-locked host, 2 pageable host (-1 when not checked).  The cross-transfer checks
 // (overlaps) are the batch's.
-mpt_status batch_check_xfer(mpt_ctx_t c, const mpt_xfer& x, int* src_kind, int* dst_kind);
+// `hints` (nullable): the arenas that the transfers before it lay in, per direction.
+struct ArenaHints {
+  size_t src[3] = {0, 0, 0}, dst[3] = {0, 0, 0};
+};
+mpt_status batch_check_xfer(mpt_ctx_t c, const mpt_xfer& x, int* src_kind, int* dst_kind, ArenaHints* hints = nullptr);
+
+// The batch's kernel has ended (mpt_batch_wait returns once every transfer is done, which is before).
+bool batch_finished(mpt_batch_t b);
 
 // Device time in ms between the timing events around a finished batch's replay (from the
 // stream reaching the replay to its end), or -1 when the batch was not timed.
@@ -197,7 +204,7 @@ struct mpt_ctx_s {
   std::vector<mpt::Arena> arenas;
   uint32_t batch_slots = 0, batch_max_xfers = 0, batch_ctas = 0, batch_tile = 0;
   // mpt_batch_submit's per-batch scratch, kept to avoid allocating per batch
-  std::vector<std::pair<uint64_t, uint64_t>> batch_spans;
+  std::vector<std::pair<uint64_t, uint64_t>> batch_spans[2];  // destinations: device, host
   std::vector<uint32_t> batch_cand;
   std::vector<uint8_t> batch_to_dma;
   uint32_t batch_dma_lanes = 0, batch_dma_items = 0;  // per direction; items per lane

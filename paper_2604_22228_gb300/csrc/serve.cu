@@ -169,7 +169,7 @@ void serve_loop(mpt_server_s* s) {
         }
         f.ndone = n;
       }
-      if (f.ndone == f.reqs.size() && mpt_batch_wait(f.batch, 0) == MPT_OK) {
+      if (f.ndone == f.reqs.size() && batch_finished(f.batch)) {
         const uint64_t t_done = steady_ns();
         const uint64_t took = t_done - f.launch_ns;
         if (!s->batch_log.empty())

@@ -73,3 +73,33 @@ def test_batch_lengths_and_mixed_directions(ctx, n, step):
         xs.append((int(r.randint(0, 9000 if n < 2000 else 700)), off, off if step == 16 else int(r.randint(0, 128)),
                    int(r.randint(0, 3))))
     _run(ctx, xs, 0xF0000 + n)
+
+
+def test_overlaps_are_found_in_any_order(ctx):
+    """Destinations that overlap one another, and sources that overlap a destination, are refused
+    wherever they stand in the batch and whatever the others' order; the same batch without the
+    offending transfer is accepted."""
+    import torch
+    dev = torch.zeros(1 << 20, dtype=torch.uint8, device="cuda")
+    host = torch.zeros(1 << 20, dtype=torch.uint8).pin_memory()
+    d, h = dev.data_ptr(), host.data_ptr()
+    d2d, h2d, d2h = mpt.MPT_D2D, mpt.MPT_H2D, mpt.MPT_D2H
+    good = [(d + 4096 * i, d + (512 << 10) + 4096 * i, 4000, d2d) for i in range(20)]
+    good += [(h + 4096 * i, d + (640 << 10) + 4096 * i, 4000, h2d) for i in range(20)]
+    good += [(d + 4096 * i, h + (512 << 10) + 4096 * i, 4000, d2h) for i in range(20)]
+    bad = [(d, d + (512 << 10) + 4096 * 7 + 3999, 2, d2d),   # the last byte of a destination
+           (h, d + (640 << 10) - 1, 2, h2d),                 # the first byte of one
+           (d, h + (512 << 10) + 4096 * 19 + 100, 5, d2h),   # inside the last one
+           (d + (512 << 10) + 4096 * 3, d + (900 << 10), 8, d2d),      # a source inside a destination
+           (h + (512 << 10) - 4, d + (900 << 10), 8, h2d),             # reaching into the first
+           (d + (512 << 10) - 4000, d + (900 << 10), 200 << 10, d2d)]  # spanning several
+    for order in (list(good), good[::-1], good[1::2] + good[::2]):
+        for x in bad:
+            for at in (0, 31, len(order)):
+                with pytest.raises(mpt.MptError) as e:
+                    mpt.mpt_batch_submit(ctx, order[:at] + [x] + order[at:])
+                assert e.value.status == mpt.MPT_EINVAL, x
+        b = mpt.mpt_batch_submit(ctx, order + [(d + (900 << 10), d + (900 << 10), 0, d2d)])
+        mpt.mpt_batch_wait(b)
+        assert mpt.mpt_batch_poll(b)[0] == len(order) + 1
+        mpt.mpt_batch_release(b)
