@@ -507,7 +507,11 @@ uint64_t mpt::batch_cta_spread_ns(mpt_batch_t b) {
   return last >= first ? last - first : 0;
 }
 
-bool mpt::batch_finished(mpt_batch_t b) { return cudaEventQuery(b->ctx->slots[b->slot].done_ev) == cudaSuccess; }
+bool mpt::batch_finished(mpt_batch_t b) {
+  mpt::BatchSlot& s = b->ctx->slots[b->slot];
+  if (!s.idle) s.idle = cudaEventQuery(s.done_ev) == cudaSuccess;
+  return s.idle;
+}
 
 float mpt::batch_gpu_ms(mpt_batch_t b) {
   const mpt::BatchSlot& s = b->ctx->slots[b->slot];
@@ -660,16 +664,17 @@ mpt_status mpt_batch_submit(mpt_ctx_t c, const mpt_xfer* xfers, size_t n, void* 
   if (st != MPT_OK) return st;
   if (n == 0 || n > c->slots[0].max_xfers)
     return fail(MPT_EINVAL, "mpt_batch_submit: %zu transfers (1..%u per batch)", n, c->slots[0].max_xfers);
-  // a free slot whose previous batch has left the GPU, else any free one
-  uint32_t si = (uint32_t)c->slots.size();
-  for (uint32_t i = 0; i < c->slots.size(); ++i) {
+  // a free slot whose previous batch is known to have left the GPU, else one that turns out to
+  // have, else any free one
+  uint32_t si = (uint32_t)c->slots.size(), busy = si;
+  for (uint32_t i = 0; i < c->slots.size() && si == c->slots.size(); ++i) {
     if (c->slots[i].held) continue;
-    if (si == c->slots.size()) si = i;
-    if (cudaEventQuery(c->slots[i].done_ev) == cudaSuccess) {
-      si = i;
-      break;
-    }
+    if (c->slots[i].idle) si = i;
+    else if (busy == c->slots.size()) busy = i;
   }
+  for (uint32_t i = busy; i < c->slots.size() && si == c->slots.size(); ++i)
+    if (!c->slots[i].held && cudaEventQuery(c->slots[i].done_ev) == cudaSuccess) si = i;
+  if (si == c->slots.size()) si = busy;
   if (si == c->slots.size()) return fail(MPT_EAGAIN, "mpt_batch_submit: every batch slot is held");
   BatchSlot& s = c->slots[si];
   // validate: direction, memory kinds, and non-overlapping destinations (Sec. 4.5: each
@@ -728,7 +733,7 @@ mpt_status mpt_batch_submit(mpt_ctx_t c, const mpt_xfer* xfers, size_t n, void* 
       return fail(MPT_EINVAL, "mpt_batch_submit: the source of transfer %zu overlaps a destination of the batch", i);
   }
   // the slot's previous batch must be done reading its table
-  CUDA_TRY(cudaEventSynchronize(s.done_ev));
+  if (!s.idle) CUDA_TRY(cudaEventSynchronize(s.done_ev));
   s.epoch++;
   if (s.epoch == 0) s.epoch = 1;
   // DMA lanes: largest eligible entries first, each to the least-loaded lane of its
@@ -839,6 +844,7 @@ mpt_status mpt_batch_submit(mpt_ctx_t c, const mpt_xfer* xfers, size_t n, void* 
   CUDA_TRY(cudaEventRecord(s.done_ev, cs));
   s.timed = timed;
   s.held = true;
+  s.idle = false;
   s.n = n;
   mpt_batch_s* b = new mpt_batch_s{c, si, s.epoch, n, host_ns()};
   *out = b;

@@ -82,6 +82,7 @@ struct BatchSlot {
   cudaEvent_t t0_ev = nullptr, t1_ev = nullptr;  // timing events around the replay (batch_timing)
   uint32_t epoch = 0;
   bool held = false;
+  bool idle = true;    // its last batch was seen to have left the GPU
   bool timed = false;  // the last replay was bracketed by t0_ev / t1_ev
   size_t n = 0;
   // DMA lanes: for each direction (D2D, H2D, D2H) `lanes` chains of `items` copy-engine
