@@ -495,7 +495,8 @@ MPT_API mpt_status mpt_batch_register(mpt_ctx_t ctx, const void* base, uint64_t 
  * (Sec. 4.5: each transfer owns its region).  The descriptor table is copied into the
  * slot, so `xfers` may be reused on return; the replay copies only the table's used bytes
  * to the device (a few hundred for a short batch) and the kernel resets its own counters,
- * so a one-transfer batch is one small copy and one kernel.  *out is owned by the caller until
+ * and a batch of at most eight transfers without lane entries is one kernel that carries the
+ * table in its launch.  *out is owned by the caller until
  * mpt_batch_release, which frees the slot.  Errors: EINVAL (bad descriptor, overlapping
  * destinations, n outside 1..max_xfers), EAGAIN (every slot held), ECUDA. */
 MPT_API mpt_status mpt_batch_submit(mpt_ctx_t ctx, const mpt_xfer* xfers, size_t n, void* stream, mpt_batch_t* out);

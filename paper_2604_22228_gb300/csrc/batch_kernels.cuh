@@ -61,6 +61,14 @@ struct BatchArgs {
   unsigned long long* host_stamps;  // device alias of page-locked [first, last] CTA start times
 };
 
+// A short batch carries its table in the kernel's arguments.
+constexpr uint32_t kInlineXfers = 8;
+struct BatchInline {
+  BatchArgs args;
+  BatchHeader hdr;
+  BatchDesc desc[kInlineXfers];
+};
+
 // Completion of one DMA-lane item: dma_map[item] is the descriptor its copy-engine node
 // moved (~0 when the item is unused); stamps its time and raises its host flag.
 __global__ void k_batch_dma_done(BatchArgs a, const uint32_t* dma_map, uint32_t item);

@@ -1,5 +1,6 @@
 """The batch kernel's tiles: sizes around the tile and line boundaries at every kind of
-alignment and direction, and batch lengths around the steps of the descriptor search.  Whole
+alignment and direction, and batch lengths around the steps of the descriptor search and the
+longest table that a launch carries.  Whole
 arenas are compared with the oracle's copies, so bytes between the transfers must stay as they
 were."""
 import numpy as np
@@ -63,7 +64,7 @@ def test_tile_and_line_edges(ctx, direction, offsets):
     _run(ctx, [(n, *offsets, direction) for n in EDGES], 0xE0000 + 64 * direction + offsets[0])
 
 
-@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 63, 64, 65, 1023, 1024, 1025, 1057, 4096])
+@pytest.mark.parametrize("n", [1, 2, 7, 8, 9, 31, 32, 33, 63, 64, 65, 1023, 1024, 1025, 1057, 4096])
 @pytest.mark.parametrize("step", [16, 1])
 def test_batch_lengths_and_mixed_directions(ctx, n, step):
     r = np.random.RandomState(n + step)
