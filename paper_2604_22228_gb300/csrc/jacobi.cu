@@ -34,7 +34,19 @@ __device__ __forceinline__ float jacobi_point(float up, float down, float left, 
   return __fmul_rn(__fadd_rn(__fadd_rn(up, down), __fadd_rn(left, right)), 0.25f);
 }
 
-__device__ __forceinline__ float4 ld4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
+// Plain loads that stay where they are written, behind the wait for the kernel ahead: that kernel
+// may still be writing the rows while this one starts, so they are no read-only data.
+__device__ __forceinline__ float4 ld4(const float* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+
+__device__ __forceinline__ float ld1(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
 
 // Both kernels cut the rows into strips of kR and give a strip of some columns to each warp.
 // The sweep is bound by memory, so a warp issues every load of its strip (kR + 2 rows) before
@@ -48,7 +60,7 @@ __device__ __forceinline__ float4 ld4(const float* p) { return __ldg(reinterpret
 // neighbours come from the adjacent lanes (shuffles); the two lanes at the warp's edges read
 // their outside neighbour from global memory.
 template <int kR>
-__global__ void __launch_bounds__(kThreads) k_jacobi_v4(const float* __restrict__ in, float* __restrict__ out,
+__global__ void __launch_bounds__(kThreads) k_jacobi_v4(const float* in, float* out,
                                                         uint32_t rows, uint64_t cols) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t nq = cols / 4;
@@ -70,7 +82,7 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_v4(const float* __restrict_
     for (int i = 0; i < kR + 2; ++i)
       if (i < 2 || (uint32_t)i < n + 2) x[i] = ld4(ip + (uint64_t)i * cols + c0);
 #pragma unroll
-    for (int i = 0; i < kR; ++i) e[i] = edge && (uint32_t)i < n ? __ldg(ip + (uint64_t)(i + 1) * cols + ec) : 0.0f;
+    for (int i = 0; i < kR; ++i) e[i] = edge && (uint32_t)i < n ? ld1(ip + (uint64_t)(i + 1) * cols + ec) : 0.0f;
 #pragma unroll
     for (int i = 0; i < kR; ++i) {
       if ((uint32_t)i >= n) break;
@@ -95,7 +107,7 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_v4(const float* __restrict_
 // warp's 32 * kG columns need a load of their own.  With one group (or one point per thread, as
 // before) too few bytes are in flight: 16384 x 16381 took 847 us, 543 with kG = 1, 359 now.
 template <int kR, int kG>
-__global__ void __launch_bounds__(kThreads) k_jacobi(const float* __restrict__ in, float* __restrict__ out,
+__global__ void __launch_bounds__(kThreads) k_jacobi(const float* in, float* out,
                                                      uint32_t rows, uint64_t cols) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t w0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x - lane) * kG;  // the warp's first column
@@ -116,9 +128,9 @@ __global__ void __launch_bounds__(kThreads) k_jacobi(const float* __restrict__ i
     for (int i = 0; i < kR + 2; ++i)
 #pragma unroll
       for (int g = 0; g < kG; ++g)
-        x[i][g] = (i < 2 || (uint32_t)i < n + 2) && c0 + 32 * g < cols ? __ldg(ip + (uint64_t)i * cols + c0 + 32 * g) : 0.0f;
+        x[i][g] = (i < 2 || (uint32_t)i < n + 2) && c0 + 32 * g < cols ? ld1(ip + (uint64_t)i * cols + c0 + 32 * g) : 0.0f;
 #pragma unroll
-    for (int i = 0; i < kR; ++i) e[i] = edge && (uint32_t)i < n ? __ldg(ip + (uint64_t)(i + 1) * cols + ec) : 0.0f;
+    for (int i = 0; i < kR; ++i) e[i] = edge && (uint32_t)i < n ? ld1(ip + (uint64_t)(i + 1) * cols + ec) : 0.0f;
 #pragma unroll
     for (int i = 0; i < kR; ++i) {
       if ((uint32_t)i >= n) break;
