@@ -10,7 +10,6 @@ namespace mpt {
 // ---- batched transfers: persistent descriptor-table kernel --------------------------
 constexpr uint32_t kDescHostDst = 1;   // destination is host memory: publish with system fences
 constexpr uint32_t kDescHostSide = 2;  // one side is host memory: coherent loads, no read-only path
-constexpr uint32_t kDescDma = 4;       // moved by a copy-engine lane, not by the kernel (ntiles 0)
 
 // Tiles come in two classes, each numbered from 0 and claimed through its own cursor: link
 // tiles (one side in host memory: they move over the host link) and device tiles (both sides

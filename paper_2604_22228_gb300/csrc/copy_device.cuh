@@ -36,15 +36,6 @@ __device__ __forceinline__ void record_invalid(uint32_t* status, uint32_t site) 
   if (status) atomicCAS(status, 0u, (site << 8) | kInvalid);
 }
 
-// Read-only path (ld.global.nc): only for data no agent writes while the kernel runs.
-__device__ __forceinline__ uint4 ld_stream(const uint4* p) {
-  uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "l"(p));
-  return v;
-}
-
 __device__ __forceinline__ uint4 ld_plain(const uint4* p) {
   uint4 v;
   asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
@@ -60,24 +51,19 @@ __device__ __forceinline__ uint4 ld_once(const uint4* p) {
   return v;
 }
 
-// 32 bytes in one instruction, for both ends 32-byte aligned.
+// 32 bytes in one instruction, for both ends 32-byte aligned.  Coherent, and not through the
+// read-only path on the device either: a kernel launched with programmatic stream serialization
+// starts while the one ahead may still be writing its source.
 struct Wide {
   uint32_t w[8];
 };
 
-template <bool kCoherent>
 __device__ __forceinline__ Wide ld_wide(const void* p) {
   Wide v;
-  if (kCoherent)
-    asm volatile("ld.global.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3]), "=r"(v.w[4]), "=r"(v.w[5]), "=r"(v.w[6]),
-                   "=r"(v.w[7])
-                 : "l"(p));
-  else
-    asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3]), "=r"(v.w[4]), "=r"(v.w[5]), "=r"(v.w[6]),
-                   "=r"(v.w[7])
-                 : "l"(p));
+  asm volatile("ld.global.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(v.w[0]), "=r"(v.w[1]), "=r"(v.w[2]), "=r"(v.w[3]), "=r"(v.w[4]), "=r"(v.w[5]), "=r"(v.w[6]),
+                 "=r"(v.w[7])
+               : "l"(p));
   return v;
 }
 
@@ -141,52 +127,6 @@ __device__ __forceinline__ uint4 shift16(const uint4& w0, const uint4& w1, uint3
       break;
   }
   return o;
-}
-
-// The whole CTA copies n bytes s -> o: bytes until o is 16-byte aligned, 16-byte words
-// (straight when s is then aligned too, else -- only if kAny -- assembled from two aligned
-// source words), and the remaining tail bytes.  Reads never leave the 16-byte blocks that
-// hold source bytes.  Without kAny the caller guarantees s and o agree modulo 16.
-template <bool kCoherent, bool kAny>
-__device__ __forceinline__ void cta_copy(const uint8_t* s, uint8_t* o, uint64_t n) {
-  const uint32_t tid = threadIdx.x, bd = blockDim.x;
-  const uint64_t head = ((16u - (uint32_t)(reinterpret_cast<uintptr_t>(o) & 15)) & 15u) < n
-                            ? ((16u - (uint32_t)(reinterpret_cast<uintptr_t>(o) & 15)) & 15u)
-                            : n;
-  if (tid < head) o[tid] = s[tid];
-  const uint8_t* s1 = s + head;
-  uint8_t* o1 = o + head;
-  const uint64_t n1 = n - head;
-  const uint64_t nv = n1 >> 4;
-  uint4* ov = reinterpret_cast<uint4*>(o1);
-  const uint32_t m = kAny ? (uint32_t)(reinterpret_cast<uintptr_t>(s1) & 15) : 0u;
-  uint64_t v = tid;
-  if (m == 0) {
-    const uint4* sv = reinterpret_cast<const uint4*>(s1);
-    for (; v + 3ull * bd < nv; v += 4ull * bd) {
-      uint4 r0, r1, r2, r3;
-      if (kCoherent) {
-        r0 = ld_plain(sv + v); r1 = ld_plain(sv + v + bd); r2 = ld_plain(sv + v + 2 * bd); r3 = ld_plain(sv + v + 3 * bd);
-      } else {
-        r0 = ld_stream(sv + v); r1 = ld_stream(sv + v + bd); r2 = ld_stream(sv + v + 2 * bd); r3 = ld_stream(sv + v + 3 * bd);
-      }
-      st_plain(ov + v, r0);
-      st_plain(ov + v + bd, r1);
-      st_plain(ov + v + 2 * bd, r2);
-      st_plain(ov + v + 3 * bd, r3);
-    }
-    for (; v < nv; v += bd) st_plain(ov + v, kCoherent ? ld_plain(sv + v) : ld_stream(sv + v));
-  } else {
-    const uint4* sw = reinterpret_cast<const uint4*>(s1 - m);
-    const uint32_t k = m >> 2, r = (m & 3u) * 8u;
-#pragma unroll 2
-    for (; v < nv; v += bd) {
-      const uint4 a0 = kCoherent ? ld_plain(sw + v) : ld_stream(sw + v);
-      const uint4 a1 = kCoherent ? ld_plain(sw + v + 1) : ld_stream(sw + v + 1);
-      st_plain(ov + v, shift16(a0, a1, k, r));
-    }
-  }
-  for (uint64_t b = (nv << 4) + tid; b < n1; b += bd) o1[b] = s1[b];
 }
 
 }  // namespace mpt

@@ -3,8 +3,8 @@
 //  k_sm_copy_vec   SM copy kernel: each CTA walks tiles of the ranges it is given, every thread
 //                  keeping kU 32-byte vectors in flight.  The device-to-device path the SMs add
 //                  next to the copy engines (Sec. 4.3's horizontal split over paths).
-//  k_zc_copy       zero-copy kernel: the same loop with coherent loads, used on mapped
-//                  page-locked host memory for host<->device transfers.
+//  k_zc_copy       zero-copy kernel: the same loop without the first tile's prefetch, used on
+//                  mapped page-locked host memory for host<->device transfers.
 //
 // The bulk-copy variant of the SM copy kernel (cp.async.bulk through shared memory) is in
 // copy_bulk.cu.
@@ -52,7 +52,7 @@ __device__ __forceinline__ void prefetch_first_tile(const Args& a) {
 // them but in a range's first and last tile.  o is 32-byte aligned.
 
 // Source and destination agree modulo 32: kU units a thread.
-template <bool kCoherent, int kU>
+template <int kU>
 __device__ __forceinline__ void copy_units(const uint8_t* s, uint8_t* o, int lo, int hi) {
   const int i0 = (int)threadIdx.x;
   s += 32 * i0;
@@ -60,7 +60,7 @@ __device__ __forceinline__ void copy_units(const uint8_t* s, uint8_t* o, int lo,
   Wide x[kU];
 #pragma unroll
   for (int u = 0; u < kU; ++u)
-    if (i0 + kVecThreads * u >= lo && i0 + kVecThreads * u < hi) x[u] = ld_wide<kCoherent>(s + kVecTile * u);
+    if (i0 + kVecThreads * u >= lo && i0 + kVecThreads * u < hi) x[u] = ld_wide(s + kVecTile * u);
 #pragma unroll
   for (int u = 0; u < kU; ++u)
     if (i0 + kVecThreads * u >= lo && i0 + kVecThreads * u < hi) st_wide(o + kVecTile * u, x[u]);
@@ -88,7 +88,7 @@ __device__ __forceinline__ void store_shifted(const Wide (&x)[kU + 1], uint8_t* 
   }
 }
 
-template <bool kCoherent, int kU>
+template <int kU>
 __device__ __forceinline__ void copy_shifted(const uint8_t* s, uint8_t* o, uint32_t m, int lo, int hi) {
   const uint32_t lane = threadIdx.x & 31u;
   const int i0 = (int)((threadIdx.x - lane) * kU + lane);
@@ -98,7 +98,7 @@ __device__ __forceinline__ void copy_shifted(const uint8_t* s, uint8_t* o, uint3
   Wide x[kU + 1];
 #pragma unroll
   for (int u = 0; u <= kU; ++u)
-    if (i0 + 32 * u >= lo && i0 + 32 * u <= last && (u < kU || lane == 0)) x[u] = ld_wide<kCoherent>(s + 1024 * u);
+    if (i0 + 32 * u >= lo && i0 + 32 * u <= last && (u < kU || lane == 0)) x[u] = ld_wide(s + 1024 * u);
   const uint32_t r = (m & 3u) * 8u;
   switch (m) {
     case 4: store_shifted<1, false, kU>(x, o, 0, lane, i0, lo, hi); return;
@@ -117,7 +117,7 @@ __device__ __forceinline__ void copy_shifted(const uint8_t* s, uint8_t* o, uint3
   }
 }
 
-template <bool kCoherent, bool kAny, int kU, typename Args>
+template <bool kAny, int kU, typename Args>
 __device__ __forceinline__ void copy_tiles(const Args& a) {
   constexpr int64_t kUnits = (int64_t)kVecThreads * kU;
   for (uint32_t t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
@@ -135,8 +135,8 @@ __device__ __forceinline__ void copy_tiles(const Args& a) {
     const int lo = u0 < 0 ? (int)-u0 : 0, hi = units - u0 < kUnits ? (int)(units - u0) : (int)kUnits;
     s += 32 * u0;
     o += 32 * u0;
-    if (kAny && d.shift) copy_shifted<kCoherent, kU>(s, o, d.shift, lo, hi);
-    else copy_units<kCoherent, kU>(s, o, lo, hi);
+    if (kAny && d.shift) copy_shifted<kU>(s, o, d.shift, lo, hi);
+    else copy_units<kU>(s, o, lo, hi);
   }
 }
 
@@ -153,13 +153,13 @@ template <int kU, bool kAny, int kN>
 __global__ void __launch_bounds__(kVecThreads, kAny ? 4 - kU : kU == 4 ? 2 : 4) k_sm_copy_vec(const __grid_constant__ CopyArgsT<kN> a) {
   prefetch_first_tile<kVecTile * kU>(a);
   pdl_enter();
-  copy_tiles<false, kAny, kU>(a);
+  copy_tiles<kAny, kU>(a);
 }
 
 template <bool kAny, int kN>
 __global__ void __launch_bounds__(kVecThreads) k_zc_copy(const __grid_constant__ CopyArgsT<kN> a) {
   pdl_enter();
-  copy_tiles<true, kAny, 4>(a);
+  copy_tiles<kAny, 4>(a);
 }
 
 // ---- host side -------------------------------------------------------------------------

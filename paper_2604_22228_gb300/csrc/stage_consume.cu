@@ -17,6 +17,45 @@
 
 namespace mpt {
 
+namespace {
+
+// The whole CTA copies n bytes s -> o: bytes until o is 16-byte aligned, 16-byte words
+// (straight when s is then aligned too, else assembled from two aligned source words), and the
+// remaining tail bytes.  Reads never leave the 16-byte blocks that hold source bytes.
+__device__ __forceinline__ void cta_copy(const uint8_t* s, uint8_t* o, uint64_t n) {
+  const uint32_t tid = threadIdx.x, bd = blockDim.x;
+  const uint64_t skew = (16u - (uint32_t)(reinterpret_cast<uintptr_t>(o) & 15)) & 15u;
+  const uint64_t head = skew < n ? skew : n;
+  if (tid < head) o[tid] = s[tid];
+  const uint8_t* s1 = s + head;
+  uint8_t* o1 = o + head;
+  const uint64_t n1 = n - head;
+  const uint64_t nv = n1 >> 4;
+  uint4* ov = reinterpret_cast<uint4*>(o1);
+  const uint32_t m = (uint32_t)(reinterpret_cast<uintptr_t>(s1) & 15);
+  uint64_t v = tid;
+  if (m == 0) {
+    const uint4* sv = reinterpret_cast<const uint4*>(s1);
+    for (; v + 3ull * bd < nv; v += 4ull * bd) {
+      const uint4 r0 = ld_plain(sv + v), r1 = ld_plain(sv + v + bd), r2 = ld_plain(sv + v + 2 * bd),
+                  r3 = ld_plain(sv + v + 3 * bd);
+      st_plain(ov + v, r0);
+      st_plain(ov + v + bd, r1);
+      st_plain(ov + v + 2 * bd, r2);
+      st_plain(ov + v + 3 * bd, r3);
+    }
+    for (; v < nv; v += bd) st_plain(ov + v, ld_plain(sv + v));
+  } else {
+    const uint4* sw = reinterpret_cast<const uint4*>(s1 - m);
+    const uint32_t k = m >> 2, r = (m & 3u) * 8u;
+#pragma unroll 2
+    for (; v < nv; v += bd) st_plain(ov + v, shift16(ld_plain(sw + v), ld_plain(sw + v + 1), k, r));
+  }
+  for (uint64_t b = (nv << 4) + tid; b < n1; b += bd) o1[b] = s1[b];
+}
+
+}  // namespace
+
 __global__ void __launch_bounds__(kVecThreads) k_stage_consume(StageArgs a) {
   __shared__ int ok;
   constexpr uint64_t kTile = kStageTile;
@@ -49,7 +88,7 @@ __global__ void __launch_bounds__(kVecThreads) k_stage_consume(StageArgs a) {
     const uint64_t off = (uint64_t)lt * kTile;
     if (off < c.bytes) {
       const uint64_t n = c.bytes - off < kTile ? c.bytes - off : kTile;
-      cta_copy<true, true>(a.stage + c.stage_off + off, a.dst + c.dst_off + off, n);
+      cta_copy(a.stage + c.stage_off + off, a.dst + c.dst_off + off, n);
     }
     __syncthreads();
     if (tid == 0) {
