@@ -861,6 +861,12 @@ mpt_status mpt_batch_submit(mpt_ctx_t c, const mpt_xfer* xfers, size_t n, void* 
     CUDA_TRY(cudaEventCreate(&s.t1_ev));
   }
   if (timed) CUDA_TRY(cudaEventRecord(s.t0_ev, cs));
+  // The launch's own status decides, not the runtime's last error, which an earlier call of the
+  // caller's may have left.  From here on the slot counts as busy: where the record of its event
+  // fails, the batch is waited for, so that a call that failed leaves nothing running on the
+  // caller's buffers and on the slot.
+  s.idle = false;
+  cudaError_t e;
   if (use_inline) {
     // no more CTAs than there are tiles for
     const uint32_t grid = (uint32_t)std::min<uint64_t>(ctas, std::max<uint64_t>(1, link_ctas + tiles[1]));
@@ -868,17 +874,22 @@ mpt_status mpt_batch_submit(mpt_ctx_t c, const mpt_xfer* xfers, size_t n, void* 
     in.args = s.args;
     in.hdr = *h;
     std::memcpy(in.desc, d, n_tiled * sizeof(BatchDesc));
-    if (gi == 0) k_batch_short<false><<<grid, kBatchThreads, 0, cs>>>(in);
-    else k_batch_short<true><<<grid, kBatchThreads, 0, cs>>>(in);
-    CUDA_TRY(cudaGetLastError());
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kBatchThreads);
+    cfg.stream = cs;
+    e = gi == 0 ? cudaLaunchKernelEx(&cfg, k_batch_short<false>, in) : cudaLaunchKernelEx(&cfg, k_batch_short<true>, in);
   } else {
-    CUDA_TRY(cudaGraphLaunch(s.exec[gi], cs));
+    e = cudaGraphLaunch(s.exec[gi], cs);
   }
-  if (timed) CUDA_TRY(cudaEventRecord(s.t1_ev, cs));
-  CUDA_TRY(cudaEventRecord(s.done_ev, cs));
+  if (e == cudaSuccess) {
+    if (timed) e = cudaEventRecord(s.t1_ev, cs);
+    if (e == cudaSuccess) e = cudaEventRecord(s.done_ev, cs);
+    if (e != cudaSuccess) cudaStreamSynchronize(cs);
+  }
+  if (e != cudaSuccess) return fail(MPT_ECUDA, "mpt_batch_submit: launch: %s", cudaGetErrorString(e));
   s.timed = timed;
   s.held = true;
-  s.idle = false;
   s.n = n;
   mpt_batch_s* b = new mpt_batch_s{c, si, s.epoch, n, host_ns()};
   *out = b;

@@ -1,0 +1,109 @@
+"""Host code of the library when a CUDA call fails, linked against a stand-in runtime
+(tests/native/fake_cudart.cpp) that fails calls on request and logs launches: no GPU needed."""
+import ctypes as C
+import os
+import shutil
+import subprocess
+
+import pytest
+
+import paper_2604_22228_gb300 as mpt
+from paper_2604_22228_gb300 import _ffi, build
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+MiB = 1 << 20
+ERROR = 700  # any error code
+
+
+@pytest.fixture(scope="module")
+def library(tmp_path_factory):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if not cxx:
+        pytest.skip("no host C++ compiler")
+    build.build()
+    objs = [os.path.join(build.OBJDIR, s + ".o") for s in build.SOURCES]
+    for s, o in zip(build.SOURCES, objs):
+        if not os.path.exists(o):
+            os.makedirs(build.OBJDIR, exist_ok=True)
+            build._compile(build._nvcc(), s)
+    include = os.path.join(os.path.dirname(os.path.dirname(build._nvcc())), "include")
+    out = str(tmp_path_factory.mktemp("fake") / "libmpt_fake.so")
+    subprocess.run([cxx, "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I", include,
+                    os.path.join(ROOT, "tests", "native", "fake_cudart.cpp"), *objs, "-ldl", "-pthread", "-o", out],
+                   check=True, capture_output=True, text=True)
+    return out
+
+
+@pytest.fixture
+def fake(library, tmp_path, monkeypatch):
+    """The stand-in's controls; the package calls the library linked against it meanwhile."""
+    path = str(tmp_path / "libmpt_fake.so")  # a copy of its own: every test starts with fresh state
+    shutil.copy(library, path)
+    monkeypatch.setattr(_ffi, "_lib", None)
+    lib = _ffi.load(path)
+    lib.fake_fail.argtypes = [C.c_char_p, C.c_int, C.c_int]
+    lib.fake_count.argtypes = lib.fake_loaded.argtypes = [C.c_char_p]
+    lib.fake_capturing.argtypes = [C.c_void_p]
+    lib.fake_launches.argtypes = [C.c_char_p, C.POINTER(C.c_uint), C.POINTER(C.c_int)]
+    return lib
+
+
+@pytest.fixture
+def ctx(fake):
+    c = mpt.mpt_ctx_create(0)
+    yield c
+    mpt.mpt_ctx_destroy(c)
+
+
+def _alloc(lib, n, host=False):
+    p = C.c_void_p()
+    assert (lib.cudaHostAlloc(C.byref(p), C.c_size_t(n), 0) if host else lib.cudaMalloc(C.byref(p), C.c_size_t(n))) == 0
+    return p.value
+
+
+def _short(lib):
+    a, b = _alloc(lib, MiB), _alloc(lib, MiB)
+    return [(a, b, 4096, mpt.MPT_D2D)]
+
+
+# ---- batches ---------------------------------------------------------------------------------
+
+def _batch(ctx, xs, stream=None):
+    b = mpt.mpt_batch_submit(ctx, xs, stream)
+    mpt.mpt_batch_wait(b)
+    mpt.mpt_batch_release(b)
+
+
+@pytest.mark.parametrize("n", [1, 8, 9])
+def test_batch_after_an_error_left_behind(fake, ctx, n):
+    """An earlier call's error, which the runtime keeps until it is asked for, is no failure of a
+    batch's launch."""
+    x = _short(fake)[0]
+    fake.fake_leave_error(ERROR)
+    _batch(ctx, [(x[0] + 4096 * i, x[1] + 4096 * i, 4096, mpt.MPT_D2D) for i in range(n)])
+
+
+@pytest.mark.parametrize("n,call,name", [(1, "launch", "k_batch_short"), (8, "cudaEventRecord", "k_batch_short"),
+                                         (9, "cudaGraphLaunch", None), (9, "cudaEventRecord", None)])
+def test_slot_after_a_failed_submission(fake, ctx, n, call, name):
+    """A submission that fails leaves nothing of its own running: what was launched before the
+    failure is waited for, and the slot serves the next batch."""
+    mpt.mpt_batch_configure(ctx, 1)
+    x = _short(fake)[0]
+    xs = [(x[0] + 4096 * i, x[1] + 4096 * i, 4096, mpt.MPT_D2D) for i in range(n)]
+
+    def launched():
+        return fake.fake_launches(name.encode(), None, None) if name else fake.fake_count(b"cudaGraphLaunch")
+
+    _batch(ctx, xs)
+    before, syncs = launched(), fake.fake_count(b"cudaStreamSynchronize")
+    fake.fake_fail(call.encode(), 0, ERROR)
+    with pytest.raises(mpt.MptError) as e:
+        mpt.mpt_batch_submit(ctx, xs)
+    assert e.value.status == mpt.MPT_ECUDA
+    if call == "cudaEventRecord":
+        assert launched() == before + 1 and fake.fake_count(b"cudaStreamSynchronize") == syncs + 1
+    queries = fake.fake_count(b"cudaEventQuery")
+    _batch(ctx, xs)
+    # the slot was asked before it was used again, beside the query of the wait
+    assert fake.fake_count(b"cudaEventQuery") >= queries + 2
