@@ -219,8 +219,12 @@ cudaError_t launch(const void* const* ptrs, const uint64_t* bytes, uint32_t n, u
   const uint32_t grid = (uint32_t)std::min<uint64_t>(tiles, ctas);
   a.per_cta = (uint32_t)tiles / grid;
   a.extra = (uint32_t)tiles % grid;
-  k_hash<kCap><<<grid, kHashThreads, 0, s>>>(a);
-  return cudaGetLastError();
+  // the launch's own status: the runtime's last error may be an earlier call's of the caller's
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kHashThreads);
+  cfg.stream = s;
+  return cudaLaunchKernelEx(&cfg, k_hash<kCap>, a);
 }
 
 // Memory kind of one range after another; ranges inside the allocation of the last query, the

@@ -107,3 +107,21 @@ def test_slot_after_a_failed_submission(fake, ctx, n, call, name):
     _batch(ctx, xs)
     # the slot was asked before it was used again, beside the query of the wait
     assert fake.fake_count(b"cudaEventQuery") >= queries + 2
+
+
+# ---- digests ---------------------------------------------------------------------------------
+
+@pytest.mark.parametrize("sizes", [[100], [MiB] * 5, [100] * 200])
+def test_digest_after_an_error_left_behind(fake, ctx, sizes):
+    a = _alloc(fake, max(sizes))
+    calls = [lambda: mpt.mpt_hash_ranges_noalloc([(a, n) for n in sizes])]
+    if len(sizes) == 1:
+        calls.append(lambda: mpt.mpt_hash_device(ctx, a, sizes[0]))
+    for call in calls:
+        fake.fake_leave_error(ERROR)
+        call()
+        fake.fake_fail(b"launch", 0, ERROR)
+        with pytest.raises(mpt.MptError) as e:
+            call()
+        assert e.value.status == mpt.MPT_ECUDA
+        call()
