@@ -498,7 +498,8 @@ MPT_API mpt_status mpt_batch_register(mpt_ctx_t ctx, const void* base, uint64_t 
  * and a batch of at most eight transfers without lane entries is one kernel that carries the
  * table in its launch.  *out is owned by the caller until
  * mpt_batch_release, which frees the slot.  Errors: EINVAL (bad descriptor, overlapping
- * destinations, n outside 1..max_xfers), EAGAIN (every slot held), ECUDA. */
+ * destinations, n outside 1..max_xfers), EAGAIN (every slot held), ECUDA (a failing call; a
+ * stream under capture). */
 MPT_API mpt_status mpt_batch_submit(mpt_ctx_t ctx, const mpt_xfer* xfers, size_t n, void* stream, mpt_batch_t* out);
 
 /* Non-blocking: number of the batch's transfers that have completed (their destination

@@ -753,6 +753,12 @@ mpt_status mpt_batch_submit(mpt_ctx_t c, const mpt_xfer* xfers, size_t n, void* 
     if ((it != spans.begin() && std::prev(it)->second > a) || (it != spans.end() && it->first < b))
       return fail(MPT_EINVAL, "mpt_batch_submit: the source of transfer %zu overlaps a destination of the batch", i);
   }
+  // a batch is launched once and waited for: a stream under capture is refused, for a captured
+  // kernel would run at the replays instead, with this batch's table and epoch
+  const cudaStream_t cs = static_cast<cudaStream_t>(stream);
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  CUDA_TRY(cudaStreamIsCapturing(cs, &cap));
+  if (cap != cudaStreamCaptureStatusNone) return fail(MPT_ECUDA, "mpt_batch_submit: the stream is under capture");
   // the slot's previous batch must be done reading its table
   if (!s.idle) CUDA_TRY(cudaEventSynchronize(s.done_ev));
   s.epoch++;
@@ -854,7 +860,6 @@ mpt_status mpt_batch_submit(mpt_ctx_t c, const mpt_xfer* xfers, size_t n, void* 
       s.table_cp_bytes[gi] = want;
     }
   }
-  const cudaStream_t cs = static_cast<cudaStream_t>(stream);
   const bool timed = c->batch_timing;
   if (timed && !s.t0_ev) {
     CUDA_TRY(cudaEventCreate(&s.t0_ev));

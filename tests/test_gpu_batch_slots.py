@@ -1,7 +1,8 @@
 """Batch slots that are used again: a ring of one slot submitted on two streams in turns, each time
 right after mpt_batch_wait saw the last flag (the kernel ahead may still be putting its counters
-back), and short batches after an error that an earlier call left behind, without the split into
-classes and with copy-engine lanes that no transfer is large enough for.  Bytes equal the oracle's
+back), and short batches after an error that an earlier call left behind, on a stream under capture
+(refused), without the split into classes and with copy-engine lanes that no transfer is large
+enough for.  Bytes equal the oracle's
 copies."""
 import numpy as np
 import pytest
@@ -70,6 +71,32 @@ def test_short_batch_after_an_error_left_behind():
         want, got = _submit_and_check(ctx, torch.cuda.Stream(), count, 4096, data, src, dst)
         assert np.array_equal(got[:count * 4096].cpu().numpy(), want)
     mpt.mpt_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("count", [1, 9])
+def test_batch_is_refused_inside_a_capture(count):
+    import torch
+    ctx = mpt.mpt_ctx_create(0)
+    mpt.mpt_batch_configure(ctx, 1)
+    data, src, dst = _buffers(9 * 4096, 0xBA7CB)
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s, capture_error_mode="relaxed"):
+        with pytest.raises(mpt.MptError):
+            _submit(ctx, s, count, src, dst)
+        dst.add_(0)
+    g.replay()
+    torch.cuda.synchronize()
+    assert not dst.any()
+    want, got = _submit_and_check(ctx, s, count, 4096, data, src, dst)
+    assert np.array_equal(got[:count * 4096].cpu().numpy(), want)
+    mpt.mpt_ctx_destroy(ctx)
+
+
+def _submit(ctx, stream, count, src, dst):
+    mpt.mpt_batch_submit(ctx, [(src.data_ptr() + 4096 * i, dst.data_ptr() + 4096 * i, 4096, mpt.MPT_D2D) for i in range(count)],
+                         stream)
 
 
 @pytest.mark.parametrize("setting", ["split off", "idle lanes"])

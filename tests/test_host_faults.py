@@ -125,3 +125,22 @@ def test_digest_after_an_error_left_behind(fake, ctx, sizes):
             call()
         assert e.value.status == mpt.MPT_ECUDA
         call()
+
+
+# ---- stream captures -------------------------------------------------------------------------
+
+@pytest.mark.parametrize("n", [1, 8, 9])
+def test_batch_is_refused_inside_a_capture(fake, ctx, n):
+    """A batch submitted to a stream under capture would run at every replay, with this batch's
+    epoch and table, and never for the caller: it is refused, and the slot stays free."""
+    mpt.mpt_batch_configure(ctx, 1)
+    x = _short(fake)[0]
+    xs = [(x[0] + 4096 * i, x[1] + 4096 * i, 4096, mpt.MPT_D2D) for i in range(n)]
+    s = _alloc(fake, 16, host=True)  # any handle
+    fake.fake_capturing(s)
+    with pytest.raises(mpt.MptError) as e:
+        mpt.mpt_batch_submit(ctx, xs, s)
+    assert e.value.status == mpt.MPT_ECUDA
+    assert fake.fake_launches(b"k_batch", None, None) == 0
+    fake.fake_capturing(None)
+    _batch(ctx, xs, s)
