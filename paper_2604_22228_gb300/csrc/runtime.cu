@@ -1354,9 +1354,11 @@ mpt_status mpt_graph_rebind(mpt_graph_t g, mpt_plan_t plan, void* dst, const voi
     if (it != c->cache.end() && it->second != g)
       return fail(MPT_EAGAIN, "mpt_graph_rebind: another cached graph already serves these addresses");
   }
-  mpt_status st = rebind(c, g, plan, dst, src);
-  if (st == MPT_OK && g->eager_plan) st = prepare_direct(c, plan, dst, src, g->direct);
+  std::vector<DirectOp> ops;  // the handle's own stay until nothing can fail any more
+  mpt_status st = g->eager_plan ? prepare_direct(c, plan, dst, src, ops) : MPT_OK;
+  if (st == MPT_OK) st = rebind(c, g, plan, dst, src);
   if (st != MPT_OK) return st;
+  g->direct.swap(ops);
   if (g->cached) {
     c->cache.erase(g->key);
     c->cache.emplace(key, g);

@@ -18,6 +18,7 @@ struct Launch {
   unsigned grid;
   bool overlap;
   void* stream;
+  void* second;  // the second pointer of the argument block: the destination of a copy kernel
 };
 struct Range {
   size_t bytes;
@@ -73,17 +74,19 @@ cudaMemoryType type_of(const void* p) {
 
 void load(const void* fn) { g_loaded[fn] = g_names[fn]; }
 
-cudaError_t launch(const char* call, const void* fn, unsigned grid, bool overlap, void* stream) {
+cudaError_t launch(const char* call, const void* fn, unsigned grid, bool overlap, void* stream, void** args) {
   const cudaError_t e = step(call);
   if (e != cudaSuccess) return e;
   load(fn);
-  g_log.push_back(Launch{g_names[fn], grid, overlap, stream});
+  void* second = nullptr;
+  if (g_names[fn].find("k_sm_copy") != std::string::npos) second = static_cast<void**>(args[0])[1];
+  g_log.push_back(Launch{g_names[fn], grid, overlap, stream, second});
   return cudaSuccess;
 }
 
-CUresult fake_cuLaunchKernelEx(const CUlaunchConfig* c, CUfunction f, void**, void**) {
-  return launch("cuLaunchKernelEx", f, c->gridDimX, c->numAttrs > 0, c->hStream) == cudaSuccess ? CUDA_SUCCESS
-                                                                                              : CUDA_ERROR_UNKNOWN;
+CUresult fake_cuLaunchKernelEx(const CUlaunchConfig* c, CUfunction f, void** args, void**) {
+  const cudaError_t e = launch("cuLaunchKernelEx", f, c->gridDimX, c->numAttrs > 0, c->hStream, args);
+  return e == cudaSuccess ? CUDA_SUCCESS : CUDA_ERROR_UNKNOWN;
 }
 
 CUresult fake_cuPointerGetAttributes(unsigned n, CUpointer_attribute* what, void** into, CUdeviceptr p) {
@@ -120,6 +123,13 @@ int fake_launches(const char* part, unsigned* grid, int* overlap) {
     }
   return n;
 }
+// Destination of the last copy kernel.
+void* fake_copied_to() {
+  void* p = nullptr;
+  for (const Launch& l : g_log)
+    if (l.second) p = l.second;
+  return p;
+}
 int fake_loaded(const char* part) {
   int n = 0;
   for (const auto& l : g_loaded) n += l.second.find(part) != std::string::npos;
@@ -152,14 +162,14 @@ cudaError_t __cudaGetKernel(cudaKernel_t* out, const void* fn) {
   *out = reinterpret_cast<cudaKernel_t>(const_cast<void*>(fn));
   return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t fn, dim3 grid, dim3, void**, size_t, cudaStream_t s) {
-  return launch("launch", fn, grid.x, false, s);
+cudaError_t __cudaLaunchKernel(cudaKernel_t fn, dim3 grid, dim3, void** args, size_t, cudaStream_t s) {
+  return launch("launch", fn, grid.x, false, s, args);
 }
-cudaError_t cudaLaunchKernel(const void* fn, dim3 grid, dim3, void**, size_t, cudaStream_t s) {
-  return launch("launch", fn, grid.x, false, s);
+cudaError_t cudaLaunchKernel(const void* fn, dim3 grid, dim3, void** args, size_t, cudaStream_t s) {
+  return launch("launch", fn, grid.x, false, s, args);
 }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* fn, void**) {
-  return launch("launch", fn, c->gridDim.x, c->numAttrs > 0, c->stream);
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* fn, void** args) {
+  return launch("launch", fn, c->gridDim.x, c->numAttrs > 0, c->stream, args);
 }
 cudaError_t cudaGetFuncBySymbol(cudaFunction_t* out, const void* fn) {
   const cudaError_t e = step("cudaGetFuncBySymbol");

@@ -44,6 +44,7 @@ def fake(library, tmp_path, monkeypatch):
     lib.fake_fail.argtypes = [C.c_char_p, C.c_int, C.c_int]
     lib.fake_count.argtypes = lib.fake_loaded.argtypes = [C.c_char_p]
     lib.fake_capturing.argtypes = [C.c_void_p]
+    lib.fake_copied_to.restype = C.c_void_p
     lib.fake_launches.argtypes = [C.c_char_p, C.POINTER(C.c_uint), C.POINTER(C.c_int)]
     return lib
 
@@ -144,3 +145,21 @@ def test_batch_is_refused_inside_a_capture(fake, ctx, n):
     assert fake.fake_launches(b"k_batch", None, None) == 0
     fake.fake_capturing(None)
     _batch(ctx, xs, s)
+
+
+# ---- handles for direct issue ----------------------------------------------------------------
+
+def test_rebind_that_fails_leaves_the_handle_as_it_was(fake, ctx):
+    n = 66 * 4096
+    old, new, src = _alloc(fake, n), _alloc(fake, n), _alloc(fake, n)
+    plan = mpt.mpt_plan(ctx, n, mpt.MPT_D2D, [(mpt.MPT_PATH_SM, 65536, n)])
+    h = mpt.mpt_prepare(ctx, plan, old, src, mpt.MPT_PREPARE_EAGER)
+    fake.fake_fail(b"cudaGetFuncBySymbol", 0, ERROR)
+    with pytest.raises(mpt.MptError):
+        mpt.mpt_graph_rebind(h, plan, new, src)
+    for k, to in ((1, old), (2, new)):
+        mpt.mpt_launch(h)
+        assert fake.fake_launches(b"k_sm_copy", None, None) == k and fake.fake_copied_to() == to
+        mpt.mpt_graph_rebind(h, plan, new, src)
+    mpt.mpt_graph_release(h)
+    mpt.mpt_plan_destroy(plan)
