@@ -649,7 +649,8 @@ MPT_API mpt_status mpt_serve_stop(mpt_server_t server);
  * out[r][c] = ((in[r-1][c] + in[r+1][c]) + (in[r][c-1] + in[r][c+1])) * 0.25, each operation
  * rounded to fp32 in that order; columns 0 and cols-1 copied; out's halo rows untouched.
  * Asynchronous on `stream` (legal inside a stream capture; outside one the launch overlaps the
- * end of the kernel before it on `stream`, as direct copies do).  Errors: EINVAL. */
+ * end of the kernel before it on `stream`, as direct copies do; MPT_PDL=0 when the process makes
+ * its first sweep turns that off).  Errors: EINVAL. */
 MPT_API mpt_status mpt_demo_jacobi_step(const float* in, float* out, uint32_t rows, uint64_t cols, void* stream);
 
 /* ---- failure detection self-test ---------------------------------------------------- */

@@ -12,6 +12,7 @@
 // reproduces it bit for bit); columns 0 and cols-1 are copied unchanged; halo rows of
 // `out` are not written.
 #include <algorithm>
+#include <cstdlib>
 
 #include "copy_device.cuh"
 #include "internal.h"
@@ -154,6 +155,18 @@ __global__ void __launch_bounds__(kThreads) k_jacobi(const float* in, float* out
   }
 }
 
+// MPT_PDL=0 turns overlapped launches off, here as for a context's direct copies; a sweep has no
+// context to ask, so the environment is read at the process's first one.
+bool overlap_allowed() {
+  static const bool allowed = [] {
+    const char* v = std::getenv("MPT_PDL");
+    if (!v || !*v) return true;
+    char* end = nullptr;
+    return std::strtoull(v, &end, 0) != 0 || *end != 0;
+  }();
+  return allowed;
+}
+
 // Blocks of 8 warps: across a row where it is wide enough, else over strips of rows too.  Outside a
 // stream capture the launch overlaps the end of the kernel ahead, as the copy kernels' does; each
 // waits for that kernel before it touches memory (a ring of four 1024 x 4096 subdomains, two
@@ -179,7 +192,7 @@ cudaError_t launch(Kernel k, uint32_t warp_cols, uint32_t strip, const float* in
   cfg.blockDim = dim3(32 * bx, by);
   cfg.stream = s;
   cfg.attrs = attr;
-  cfg.numAttrs = cap == cudaStreamCaptureStatusNone ? 1 : 0;
+  cfg.numAttrs = cap == cudaStreamCaptureStatusNone && overlap_allowed() ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, k, in, out, rows, cols);
 }
 

@@ -163,3 +163,29 @@ def test_rebind_that_fails_leaves_the_handle_as_it_was(fake, ctx):
         mpt.mpt_graph_rebind(h, plan, new, src)
     mpt.mpt_graph_release(h)
     mpt.mpt_plan_destroy(plan)
+
+
+# ---- overlapped launches ---------------------------------------------------------------------
+
+@pytest.mark.parametrize("value,overlap", [(None, 1), ("1", 1), ("0", 0), ("0x0", 0), ("", 1)])
+@pytest.mark.parametrize("cols", [64, 63])
+def test_stencil_follows_the_overlap_switch(fake, monkeypatch, value, overlap, cols):
+    """MPT_PDL=0 turns overlapped launches off for the stencil's sweeps too, as for the contexts'
+    direct copies."""
+    monkeypatch.delenv("MPT_PDL", raising=False)
+    if value is not None:
+        monkeypatch.setenv("MPT_PDL", value)
+    a, b = _alloc(fake, MiB), _alloc(fake, MiB)
+    mpt.mpt_demo_jacobi_step(a, b, 4, cols)
+    got = C.c_int(-1)
+    assert fake.fake_launches(b"k_jacobi", None, C.byref(got)) == 1 and got.value == overlap
+    s = _alloc(fake, 16, host=True)
+    fake.fake_capturing(s)
+    mpt.mpt_demo_jacobi_step(a, b, 4, cols, s)
+    assert fake.fake_launches(b"k_jacobi", None, C.byref(got)) == 2 and got.value == 0
+    n = 4096
+    c = mpt.mpt_ctx_create(0)
+    plan = mpt.mpt_plan(c, n, mpt.MPT_D2D, [(mpt.MPT_PATH_SM, 65536, n)])
+    mpt.mpt_launch_eager(c, plan, b, a)
+    assert fake.fake_launches(b"k_sm_copy", None, C.byref(got)) == 1 and got.value == overlap
+    mpt.mpt_ctx_destroy(c)
