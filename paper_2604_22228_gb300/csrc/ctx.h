@@ -168,8 +168,13 @@ struct mpt_ctx_s {
   bool pageable = false;              // the GPU reaches pageable host memory (coherent host)
   uint32_t* d_status = nullptr;       // device status word
   unsigned long long* d_hash = nullptr;  // digest accumulator and, behind it, a count of CTAs; zero between calls
-  unsigned long long* h_hash = nullptr;  // page-locked: the digest as the kernel delivers it
-  unsigned long long* h_hash_dev = nullptr;
+  // Where the kernel delivers a digest: a host word, here in the context where the GPU reaches
+  // pageable memory, page-locked elsewhere, and its device address
+  struct alignas(64) {
+    unsigned long long word = 0;
+  } hash_line;
+  unsigned long long* h_hash = &hash_line.word;
+  unsigned long long* h_hash_dev = &hash_line.word;
   uint64_t* d_wait_ns = nullptr;      // device word: wait limit of the staged consumer's flag waits
   mpt::EagerLane lane[MPT_MAX_PATHS];
   cudaEvent_t fork = nullptr;

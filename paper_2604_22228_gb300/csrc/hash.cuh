@@ -6,7 +6,7 @@
 namespace mpt {
 
 // Where the digest of a single range goes when the kernel delivers it itself: `result` is the
-// device address of a page-locked host word, `count` a device word.  The accumulator and the
+// device address of a host word, `count` a device word.  The accumulator and the
 // count are zero between launches (the kernel leaves them so).
 struct HashResult {
   unsigned long long* result;

@@ -189,3 +189,15 @@ def test_stencil_follows_the_overlap_switch(fake, monkeypatch, value, overlap, c
     mpt.mpt_launch_eager(c, plan, b, a)
     assert fake.fake_launches(b"k_sm_copy", None, C.byref(got)) == 1 and got.value == overlap
     mpt.mpt_ctx_destroy(c)
+
+
+# ---- contexts --------------------------------------------------------------------------------
+
+def test_context_page_locks_no_memory_for_digests(fake):
+    """Page-locking costs a tenth of a millisecond, which a program that creates a context and
+    asks for no digest must not pay, nor one that asks for its first."""
+    c = mpt.mpt_ctx_create(0)
+    assert fake.fake_count(b"cudaHostAlloc") == 0
+    mpt.mpt_hash_device(c, _alloc(fake, 4096), 4096)
+    assert fake.fake_count(b"cudaHostAlloc") == 0
+    mpt.mpt_ctx_destroy(c)
