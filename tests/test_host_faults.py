@@ -201,3 +201,15 @@ def test_context_page_locks_no_memory_for_digests(fake):
     mpt.mpt_hash_device(c, _alloc(fake, 4096), 4096)
     assert fake.fake_count(b"cudaHostAlloc") == 0
     mpt.mpt_ctx_destroy(c)
+
+
+@pytest.mark.parametrize("n", [1, 9])
+def test_ring_loads_its_kernels(fake, ctx, n):
+    """A ring's kernels are loaded when it is built, not by the first batch that needs one."""
+    mpt.mpt_batch_configure(ctx)
+    loaded = fake.fake_loaded(b"")
+    assert fake.fake_loaded(b"k_batch") >= 4
+    x = _short(fake)[0]
+    for shift in (0, 1):
+        _batch(ctx, [(x[0] + 4096 * i + shift, x[1] + 4096 * i, 4000, mpt.MPT_D2D) for i in range(n)])
+    assert fake.fake_loaded(b"") == loaded
