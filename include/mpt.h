@@ -452,9 +452,9 @@ MPT_API mpt_status mpt_batch_configure_dma(mpt_ctx_t ctx, uint32_t lanes, uint32
 
 /* Batch autotuner (CTA count, tile size and DMA lanes chosen by measurement).  Runs the representative
  * batch `xfers` (n entries; their destinations are written) `reps` times (0 = 3) under each
- * candidate setting -- kernel CTAs in {1, 2, 3} x SMs, tile bytes in {64, 128, 256, 512,
- * 1024} KiB, DMA lanes off or 2 per direction for entries of at least 4 MiB -- and keeps the
- * best: objective MPT_BATCH_TUNE_TIME the shortest median batch, MPT_BATCH_TUNE_P99 the
+ * candidate setting -- kernel CTAs in {1, 2} x SMs, tile bytes in {64, 128, 256, 512,
+ * 1024} KiB, DMA lanes off, or 2 per direction for entries of at least 4 MiB or 1 MiB -- and keeps
+ * the best: objective MPT_BATCH_TUNE_TIME the shortest median batch, MPT_BATCH_TUNE_P99 the
  * lowest median p99 entry completion time (device clock, from the kernel's start).  The
  * chosen setting is applied to the context (as mpt_batch_configure and
  * mpt_batch_configure_dma would) and written to *out (nullable).  Blocking.  Errors: EINVAL,

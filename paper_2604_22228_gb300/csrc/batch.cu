@@ -596,9 +596,11 @@ mpt_status mpt_batch_tune(mpt_ctx_t c, const mpt_xfer* xfers, size_t n, uint32_t
     uint64_t min;
   };
   std::vector<Setting> cand;
-  for (uint32_t k : {1u, 2u, 3u})
+  static_assert(kBatchCtasPerSm == 2, "CTAs per SM that a batch's grid can have");
+  for (uint32_t k : {1u, 2u})
     for (uint32_t tile : {64u << 10, 128u << 10, 256u << 10, 512u << 10, 1024u << 10})
-      for (uint32_t lanes : {0u, 2u}) cand.push_back(Setting{k * sms, tile, lanes, lanes ? 8u : 0u, lanes ? 4ull << 20 : 0});
+      for (uint64_t min : {0ull, 4ull << 20, 1ull << 20})  // no lanes, or two for entries that large
+        cand.push_back(Setting{k * sms, tile, min ? 2u : 0u, min ? 8u : 0u, min});
   const uint32_t keep_slots = c->batch_slots, keep_max = c->batch_max_xfers;
   std::vector<uint64_t> t(n);
   const cudaStream_t cs = static_cast<cudaStream_t>(stream);

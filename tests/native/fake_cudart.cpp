@@ -264,7 +264,12 @@ cudaError_t cudaEventDestroy(cudaEvent_t e) { return std::free(e), cudaSuccess; 
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return step("cudaEventRecord"); }
 cudaError_t cudaEventQuery(cudaEvent_t) { return step("cudaEventQuery"); }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return step("cudaEventSynchronize"); }
-cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { return *ms = 0.001f, step("cudaEventElapsedTime"); }
+// every measurement is shorter than the one before it
+cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) {
+  const cudaError_t e = step("cudaEventElapsedTime");
+  *ms = 1.0f / (float)g_count["cudaEventElapsedTime"];
+  return e;
+}
 
 // ---- graphs ------------------------------------------------------------------------------
 cudaError_t cudaGraphCreate(cudaGraph_t* g, unsigned) { return handle("cudaGraphCreate", g); }

@@ -213,3 +213,16 @@ def test_ring_loads_its_kernels(fake, ctx, n):
     for shift in (0, 1):
         _batch(ctx, [(x[0] + 4096 * i + shift, x[1] + 4096 * i, 4000, mpt.MPT_D2D) for i in range(n)])
     assert fake.fake_loaded(b"") == loaded
+
+
+def test_batch_tune_reports_a_grid_that_runs(fake, ctx):
+    """The last setting measured is the fastest here; what is reported and applied is what its
+    kernels ran with, at most two CTAs per SM."""
+    x = _short(fake)[0]
+    xs = [(x[0] + 4096 * i, x[1] + 4096 * i, 4000, mpt.MPT_D2D) for i in range(4)]
+    r = mpt.mpt_batch_tune(ctx, xs, mpt.MPT_BATCH_TUNE_TIME, 1)
+    assert r["candidates"] == 30 and r["ctas"] == 2 * 152
+    _batch(ctx, [(x[0] + 8192 * i, x[1] + 8192 * i, 8192, mpt.MPT_D2D) for i in range(8)])
+    ran = C.c_uint()
+    fake.fake_launches(b"k_batch_short", C.byref(ran), None)
+    assert ran.value <= r["ctas"]
