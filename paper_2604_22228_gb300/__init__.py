@@ -162,7 +162,9 @@ def mpt_prepare(ctx: int, plan: int, dst, src, mode: int = MPT_PREPARE_AUTO) -> 
 
 
 def mpt_launch(graph: int, stream=None) -> None:
-    st = (_ffi._lib or lib()).mpt_launch(graph, None if stream is None else getattr(stream, "cuda_stream", stream))
+    if stream is not None and not isinstance(stream, int):
+        stream = stream.cuda_stream
+    st = (_ffi._lib or lib()).mpt_launch(graph, stream)
     if st != MPT_OK:
         _check(st, "mpt_launch")
 

@@ -226,3 +226,21 @@ def test_batch_tune_reports_a_grid_that_runs(fake, ctx):
     ran = C.c_uint()
     fake.fake_launches(b"k_batch_short", C.byref(ran), None)
     assert ran.value <= r["ctas"]
+
+
+def test_launch_takes_streams_only(fake, ctx):
+    """A stream is an int, None or an object with cuda_stream; anything else is refused before it
+    is taken for a pointer."""
+    n = 4096
+    plan = mpt.mpt_plan(ctx, n, mpt.MPT_D2D, [(mpt.MPT_PATH_SM, 65536, n)])
+    h = mpt.mpt_prepare(ctx, plan, _alloc(fake, n), _alloc(fake, n), mpt.MPT_PREPARE_EAGER)
+
+    class Stream:
+        cuda_stream = 0
+
+    for good in (None, 0, Stream()):
+        mpt.mpt_launch(h, good)
+    for bad in (b"stream", "stream", C.c_void_p(64)):
+        with pytest.raises(AttributeError):
+            mpt.mpt_launch(h, bad)
+    assert fake.fake_launches(b"k_sm_copy", None, None) == 3
