@@ -49,3 +49,24 @@ def test_device_and_host_ranges_in_one_call():
     at = [(70000 * i + i) for i in range(12)]
     got = mpt.mpt_hash_ranges_noalloc([((pinned if k else dev).data_ptr() + a, n) for k, a, n in zip(kinds, at, sizes)])
     assert got == [T.hash64(host[a:a + n]) for a, n in zip(at, sizes)]
+
+
+def test_large_device_and_host_ranges_in_one_call():
+    """Above 1 MiB a call asks where its ranges lie: launches of their own for each run of
+    neighbours of one kind, those over host memory by a small grid whose CTAs take several tiles
+    each, off 16-byte boundaries as well."""
+    import torch
+    size = 5 << 20
+    host = payload.fill("u8", 0x5EED000D, 3 * size)
+    pinned = torch.from_numpy(host).pin_memory()
+    dev = pinned.cuda()
+    ranges = [("dev", 0, 400001), ("host", 16, size), ("host", size + 5, size - 9), ("dev", size + 3, size), ("host", 7, 0),
+              ("pageable", 2 * size + 1, 3 * TILE * 32 + 11), ("dev", 0, 0), ("dev", 2 * size, 100), ("host", 1, 33)]
+    at = {"dev": dev.data_ptr(), "host": pinned.data_ptr(), "pageable": host.ctypes.data}
+    ctx = mpt.mpt_ctx_create(0)
+    if not mpt.mpt_ctx_info(ctx)["pageable_access"]:
+        ranges = [r for r in ranges if r[0] != "pageable"]
+    want = [T.hash64(host[o:o + n]) for _, o, n in ranges]
+    assert mpt.mpt_hash_ranges_noalloc([(at[k] + o, n) for k, o, n in ranges]) == want
+    assert [mpt.mpt_hash_device(ctx, at[k] + o, n) for k, o, n in ranges] == want
+    mpt.mpt_ctx_destroy(ctx)
