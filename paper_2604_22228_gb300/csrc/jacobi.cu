@@ -27,9 +27,17 @@ constexpr uint32_t kThreads = 256;
 // 400 MB of buffers), 16-byte rows at kR = 2 / 4 / 8: 512 x 1024 points 1.89 / 1.99 / 2.35;
 // 1024 x 1024 2.81 / 2.53 / 2.75; 2048 x 2048 5.43 / 4.84 / 5.53; 2048 x 4096 8.90 / 8.10 /
 // 8.15; 4096 x 4096 22.9 / 20.9 / 19.2; 8 x 16 Mi 223 / 189 / 173 (kR = 16: 181).  Other rows
-// at kR x kG = 1x1 / 2x4 / 4x4: 63 x 65 1.64 / 1.92 / 2.10; 255 x 1023 2.45 / 2.10 / 2.40;
-// 2047 x 2047 16.1 / 7.33 / 6.80; 2 x (1 Mi + 1) 9.61 / 5.70 / 6.62.
-constexpr uint64_t kTinyGrid = 1ull << 16, kSmallGrid = 3ull << 18, kLargeGrid = 1ull << 23;
+// with a point per thread and at kR x kG = 2x4 / 4x4: 64 x 33 1.18 / 1.68 / -; 1000 x 97 1.57 / 1.94
+// / -; 1000 x 193 1.86 / 1.99 / -; 300 x 1023 2.11 / 2.08 / -; 500 x 513 2.40 / 2.04 / -;
+// 2047 x 2047 - / 7.33 / 6.80; 2 x (1 Mi + 1) - / 5.70 / 6.62.
+constexpr uint64_t kTinyGrid = 3ull << 16, kSmallGrid = 3ull << 18, kLargeGrid = 1ull << 23;
+
+// Rows of at most 32 columns leave most of a warp's 128 idle, and with many of them it is the count
+// of warps that costs: one group of columns and tall strips there (us a sweep at kR x kG = 8x1 /
+// 4x4: 100,000 x 3 6.7 / 13.8; 2,000,000 x 3 103 / 240; 2,000,000 x 25 127 / 273; with a point per
+// thread, as in the first layout, 13.9, 119 and 232).
+constexpr uint64_t kNarrow = 32;
+constexpr uint32_t kNarrowRows = 4096;
 
 __device__ __forceinline__ float jacobi_point(float up, float down, float left, float right) {
   return __fmul_rn(__fadd_rn(__fadd_rn(up, down), __fadd_rn(left, right)), 0.25f);
@@ -100,6 +108,20 @@ __global__ void __launch_bounds__(kThreads) k_jacobi_v4(const float* in, float* 
       o.w = c0 + 4 == cols ? mid.w : jacobi_point(up.w, down.w, mid.z, right);
       if (active) *reinterpret_cast<float4*>(out + (uint64_t)(r0 + i + 1) * cols + c0) = o;
     }
+  }
+}
+
+// Small grids of any column count or alignment: a point per thread.  Their time is the latency of
+// one chain of loads, which strips with their shuffles make longer (1000 x 97, sweeps following
+// each other in a graph: 1.57 us, 1.99 as strips of two rows).
+__global__ void __launch_bounds__(kThreads) k_jacobi_point(const float* in, float* out, uint32_t rows, uint64_t cols) {
+  const uint64_t c = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_enter();
+  if (c >= cols) return;
+  for (uint32_t r = blockIdx.y * blockDim.y + threadIdx.y; r < rows; r += gridDim.y * blockDim.y) {
+    const float* p = in + (uint64_t)(r + 1) * cols + c;
+    out[(uint64_t)(r + 1) * cols + c] =
+        c == 0 || c + 1 == cols ? ld1(p) : jacobi_point(ld1(p - cols), ld1(p + cols), ld1(p - 1), ld1(p + 1));
   }
 }
 
@@ -216,7 +238,8 @@ extern "C" MPT_API mpt_status mpt_demo_jacobi_step(const float* in, float* out, 
     else if (rows <= 4 || points < kLargeGrid) e = launch(k_jacobi_v4<4>, 128, 4, in, out, rows, cols, s);
     else e = launch(k_jacobi_v4<8>, 128, 8, in, out, rows, cols, s);
   } else {
-    if (points < kTinyGrid) e = launch(k_jacobi<1, 1>, 32, 1, in, out, rows, cols, s);
+    if (cols <= kNarrow && rows >= kNarrowRows) e = launch(k_jacobi<8, 1>, 32, 8, in, out, rows, cols, s);
+    else if (points < kTinyGrid) e = launch(k_jacobi_point, 32, 1, in, out, rows, cols, s);
     else if (rows <= 3 || points < kSmallGrid) e = launch(k_jacobi<2, 4>, 128, 2, in, out, rows, cols, s);
     else e = launch(k_jacobi<4, 4>, 128, 4, in, out, rows, cols, s);
   }

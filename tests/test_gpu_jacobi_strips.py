@@ -67,3 +67,12 @@ def test_chain_of_sweeps_and_copies(rows, cols):
         mpt.mpt_graph_release(h)
     mpt.mpt_plan_destroy(plan)
     mpt.mpt_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("rows,cols", [(191, 1029), (192, 1025), (1, 196607), (70000, 2), (4095, 31), (4096, 32), (4097, 31), (4103, 17),
+                                       (4096, 33), (65541, 5), (600001, 3)])
+@pytest.mark.parametrize("offset", [0, 1])
+def test_small_and_narrow_grids(rows, cols, offset):
+    """Around the grid size up to which a thread takes a point, and rows of at most 32 columns in
+    tall strips, more of them than a grid has blocks across too."""
+    test_sweep_at_strip_edges(rows, cols, offset)
