@@ -162,9 +162,9 @@ def mpt_prepare(ctx: int, plan: int, dst, src, mode: int = MPT_PREPARE_AUTO) -> 
 
 
 def mpt_launch(graph: int, stream=None) -> None:
-    if stream is not None and not isinstance(stream, int):
-        stream = stream.cuda_stream
-    st = (_ffi._lib or lib()).mpt_launch(graph, stream)
+    # (the handle of a stream object in one step; an int, or a stream whose handle is 0, in two)
+    s = None if stream is None else getattr(stream, "cuda_stream", None) or _stream(stream)
+    st = (_ffi._lib or lib()).mpt_launch(graph, s)
     if st != MPT_OK:
         _check(st, "mpt_launch")
 
