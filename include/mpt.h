@@ -98,16 +98,17 @@ typedef enum { MPT_MODE_GRAPH = 0, MPT_MODE_EAGER = 1 } mpt_mode;
 #define MPT_MODE_DUPLEX 0x20u
 
 /* mpt_path_spec.flags for SM-kernel paths: which copy kernel variant to run. */
-#define MPT_SM_VEC128 0u   /* vector loads/stores, grid-stride over tiles of 16, 32 or 64 KiB by
-                              the message's size and the grid */
+#define MPT_SM_VEC128 0u   /* vector loads/stores, grid-stride over tiles of 8 to 64 KiB by the
+                              message's size and the grid */
 #define MPT_SM_BULK 1u     /* cp.async.bulk global->shared->global ring per CTA */
 /* Ring configurations of the MPT_SM_BULK kernel, chosen per context by MPT_BULK_CONFIG=i
  * (0 <= i < MPT_BULK_CONFIGS, default 3) at context creation.  Stages x stage bytes, CTAs per SM:
  * 0: 4 x 48 KiB, 1; 1: as 0 with an L2 evict-first policy; 2: 3 x 64 KiB, 1; 3: 2 x 48 KiB, 2;
  * 4: as 3 with an L2 evict-first policy; 5: 3 x 32 KiB, 2; 6: 8 x 24 KiB, 1. */
 #define MPT_BULK_CONFIGS 7u
-#define MPT_SM_TILE8K 2u   /* VEC128 over its smallest tiles (16 KiB) whatever the size
-                              (BULK takes precedence when both are set) */
+#define MPT_SM_TILE8K 2u   /* VEC128 over small tiles whatever the size: 16 KiB beyond 1 MiB (32 or 64 where
+                              source and destination differ modulo 32; BULK takes precedence
+                              when both are set) */
 /* mpt_path_spec.flags for MPT_PATH_HS in H2D/D2H: host-thread staging.  The host side of each
  * chunk is a CPU copy, by the context's pool of host threads, between the caller's host buffer
  * and a page-locked slot; the device side is a copy-engine hop between the slot and device

@@ -10,13 +10,17 @@ namespace mpt {
 
 constexpr int kInlineRanges = 16;     // ranges carried by value in one launch
 constexpr int kVecThreads = 512;      // block size of the vector copy kernels
-constexpr uint32_t kVecTile = kVecThreads * 32;  // tile bytes at one 32-byte load per thread
+constexpr uint32_t kVecTile = kVecThreads * 32;  // tile bytes at 32 bytes per thread
 constexpr int kBulkThreads = 64;      // bulk kernel block: a producer warp and a consumer warp
 
+// What the vector kernels move ranges in: units of 32 bytes, where source and destination agree
+// modulo 32; words of 16, where they agree modulo 16; or units put together from two of the
+// source's (kMoveShifted).
+constexpr uint32_t kMoveUnits = 0, kMoveWords = 1, kMoveShifted = 2;
+
 // One contiguous range to copy: src + src_off -> dst + dst_off, `bytes` long.
-// head: bytes copied singly until the destination is aligned to a unit, 32 bytes for the vector
-// kernels and 16 for the bulk kernel; shift: source minus destination address modulo a unit -- 0
-// when they agree, else each destination unit is assembled from two source units.
+// head: bytes copied singly until the destination is aligned to a unit or word; shift: source minus
+// destination address modulo that -- 0 when they agree.
 struct RangeDesc {
   uint64_t src_off;
   uint64_t dst_off;
@@ -31,7 +35,7 @@ struct CopyArgsT {
   const uint8_t* src;
   uint8_t* dst;
   uint32_t* status;                      // device status word (bounded waits)
-  uint32_t any_shift;                    // vector kernels: some range has shift != 0
+  uint32_t move;                         // vector kernels: kMoveUnits, kMoveWords or kMoveShifted
   uint32_t src_lines;                    // tiles begin on lines of the source, not of the destination
   uint32_t nranges;
   uint32_t ntiles;                       // sum of tiles over ranges
@@ -43,7 +47,7 @@ struct CopyArgsT {
 using CopyArgs = CopyArgsT<kInlineRanges>;
 
 // Fill `a` for up to kInlineRanges ranges with the tiling of `variant` (0 vec128,
-// 1 bulk in configuration bulk_cfg (bulk_config.h), 2 zero-copy, 3 vec128 with its smallest tiles)
+// 1 bulk in configuration bulk_cfg (bulk_config.h), 2 zero-copy, 3 vec128 with small tiles)
 // for a grid of at most `ctas` on `sms` SMs.  src_lines: the source is the host side of a
 // zero-copy launch.  Returns kArgsOk, kArgsNeedVec when a bulk launch must fall back to vec128
 // (source and destination differ modulo 16, which cp.async.bulk cannot copy), or kArgsTooLarge.

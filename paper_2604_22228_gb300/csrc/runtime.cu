@@ -193,7 +193,7 @@ struct CopyParams {
   CopyParams(int variant, CopyArgs& a) {
     p[0] = &a;
     if (variant == 1 || a.nranges != 1) return;
-    one = CopyArgsT<1>{a.src, a.dst, a.status, a.any_shift, a.src_lines, 1, a.ntiles, a.bulk_cfg, a.piece,
+    one = CopyArgsT<1>{a.src, a.dst, a.status, a.move, a.src_lines, 1, a.ntiles, a.bulk_cfg, a.piece,
                        {0, a.tile_start[1]}, {a.r[0]}};
     p[0] = &one;
   }

@@ -110,3 +110,20 @@ def test_direct_issue_handle_retargeted(ctx, paths):
     assert np.array_equal(dst.numpy(), T.copy(data))
     mpt.mpt_graph_release(h)
     mpt.mpt_plan_destroy(plan)
+
+
+MOVES = [8 * KiB - 1, 8 * KiB + 17, 16 * KiB, 16 * KiB + 1, 1024 * KiB - 16, 1024 * KiB, 1024 * KiB + 1, 1024 * KiB + 47,
+         152 * 16 * KiB, 152 * 16 * KiB + 1, 152 * 32 * KiB - 5, 152 * 32 * KiB + 64]
+
+
+@pytest.mark.parametrize("offsets", [(0, 0), (0, 16), (16, 0), (112, 96), (48, 48), (5, 0), (17, 1)], ids=lambda o: f"{o[0]}_{o[1]}")
+@pytest.mark.parametrize("variant", [mpt.MPT_SM_VEC128, mpt.MPT_SM_TILE8K], ids=["vec", "small_tiles"])
+def test_words_and_units(ctx, variant, offsets):
+    """Both sides of the sizes at which words give way to units and tiles grow, on grids of one
+    CTA to many, with source and destination agreeing modulo 32, 16 or not."""
+    for n in MOVES:
+        for ctas in (0, 1, 16, 152):
+            _check(ctx, n, *offsets, ("dev", "dev"), variant, ctas)
+    for where in (("host", "dev"), ("dev", "host")):
+        for n in MOVES[1:8:2]:
+            _check(ctx, n, *offsets, where, variant, 0)
