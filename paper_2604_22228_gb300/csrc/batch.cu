@@ -478,7 +478,7 @@ mpt_status batch_setup(mpt_ctx_t c) {
     c->batch_dma_min = std::max<uint64_t>(16, env_or("MPT_BATCH_DMA_MIN", 4ull << 20));
   }
   // the short batches' kernels are in no graph that would load them: without this the first short
-  // batch of a process does (its submission 15.6 us instead of 7)
+  // batch of a process does (its submission 46 us instead of 33; off 16-byte boundaries 19, not 7)
   for (const void* fn : {reinterpret_cast<const void*>(&k_batch_short<false>), reinterpret_cast<const void*>(&k_batch_short<true>)}) {
     cudaFuncAttributes attr;
     CUDA_TRY(cudaFuncGetAttributes(&attr, fn));

@@ -7,14 +7,15 @@
 // thread holds four 16-byte vectors of a tile and loads the next tile's before it mixes them.
 // With 8-byte loads one at a time and a launch per range, as before, too few bytes were in
 // flight (1.7 TB/s on 32 MiB) and every launch cost 4 us: 64 ranges of 4 KiB to 64 MiB (302 MB)
-// took 443 us a call, now 93 (the kernel 63, from a cold L2 and with its launch; HBM time 44);
+// took 448 us a call, now 92 (the kernel 53 to 54 from a cold L2; its bytes at 6.76 TB/s 45);
 // 1 GiB takes 174 us (6.2 TB/s), 206 off a 16-byte boundary.  Measured against it, 1 GiB
 // aligned / not: loads not ahead of the mixing 191 / 273 (64 registers), two vectors a tile
 // 175 / 217, 64 registers instead of 80 173 / 277 (spills), 8 CTAs per SM 177 / 210.
 //
 // A call with one range (mpt_hash_device) is bound by its round trip: the last CTA writes the sum
 // to host memory and puts the accumulator back to zero, instead of a memset before
-// and a copy after the kernel: 16 B to 64 KiB 16.7 -> 11.9 us a call, 8 MiB 23.5 -> 15.2.
+// and a copy after the kernel: 16 B to 4 KiB 17.1 -> 12.0 us a call, 64 KiB
+// 17.0 -> 13.5, 8 MiB 19.8 -> 14.8.
 #include "hash.cuh"
 
 #include <cuda.h>
@@ -39,7 +40,7 @@ constexpr uint32_t kHashHostCtas = 32;
 constexpr uint64_t kGamma = 0x9E3779B97F4A7C15ull;
 
 // kCap ranges by value: a launch copies its whole argument, so one range alone takes the small
-// one; 160 ranges fill the 4 KiB that a launch's arguments may take on any path.
+// one; 160 ranges are 3.2 KiB of the 4 that a launch's arguments may take on any path.
 template <int kCap>
 struct HashArgs {
   uint32_t n;

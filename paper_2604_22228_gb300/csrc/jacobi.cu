@@ -62,8 +62,9 @@ __device__ __forceinline__ float ld1(const float* p) {
 // the first point is computed: that keeps enough bytes in flight, each row is read once from
 // HBM (the rows two strips share come from L2), and a grid of any aspect ratio fills the SMs.
 // One thread walking down all rows of its columns, the layout before, left the GPU to the 4
-// blocks that the width gives a 1024 x 4096 subdomain: 244 us a sweep against 4.9 us now
-// (HBM time at 6.8 TB/s: 4.9 us; 16384 x 16384: 8508 us against 303, floor 316).
+// blocks that the width gives a 1024 x 4096 subdomain: 514 us a sweep over grids of 400 MB in
+// turns and 243 over one that stays in L2, against 6.9 and 4.3 now (its bytes at 6.76 TB/s: 5.0 us);
+// 16384 x 16384 8385 us against 302 (317).
 
 // 16-byte aligned rows: a lane owns four columns as one float4, a warp 128.  Horizontal
 // neighbours come from the adjacent lanes (shuffles); the two lanes at the warp's edges read
