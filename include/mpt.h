@@ -158,7 +158,7 @@ typedef struct {
  * instantiation; launch is timed by the caller). */
 typedef struct {
   uint32_t nodes;          /* graph nodes, every kind */
-  uint32_t memcpy_nodes;
+  uint32_t memcpy_nodes;   /* over the host link neighbouring chunks of a path are one, in one chain */
   uint32_t kernel_nodes;
   uint32_t memset_nodes;
   double create_us;        /* cudaGraphCreate */
